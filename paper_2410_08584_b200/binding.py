@@ -1,11 +1,13 @@
-"""ctypes binding of libzipvl.so -- argument marshalling only.
+"""Binding of libzipvl.so -- argument marshalling only.
 
 Each function has the name of the C entry point it calls (see include/zipvl.h)
 and does nothing but turn torch tensors into pointers, allocate outputs the
 caller did not pass (torch is used for device memory and streams only) and
-raise ``ZipvlError`` on a non-zero status.  Every step of the path runs in the
-library's CUDA kernels; there is no fallback: if the library cannot be loaded
-the first call raises.
+raise ``ZipvlError`` on a non-zero status.  The calls of the hot path hand their
+arguments to the extension module ``_native`` (csrc/binding.cpp), which reads the
+tensors' fields without Python objects in between; the rest goes through ctypes.
+Every step of the path runs in the library's CUDA kernels; there is no fallback: if
+the library or the module cannot be loaded the first call raises.
 """
 import ctypes as C
 import os
@@ -123,6 +125,23 @@ def load():
     return lib
 
 
+_native = None
+
+
+def _load_native():
+    """The extension module, next to libzipvl.so and built with it."""
+    global _native
+    load()
+    try:
+        from . import _native as module
+    except ImportError as e:
+        raise ImportError(f"{HERE}/_native.so cannot be loaded ({e}): run `python -m paper_2410_08584_b200.build` "
+                          "(there is no fallback path)") from e
+    module.set_error_class(ZipvlError)
+    _native = module
+    return module
+
+
 def _check(status):
     if status != 0:
         raise ZipvlError(status, load().zipvl_last_error().decode())
@@ -147,25 +166,12 @@ def _stream(stream):
     return C.c_void_p(s.cuda_stream)
 
 
-def _token_strided(t):
-    """[L, H, d] with contiguous (H, d) rows and any token stride >= H*d (a slice of a fused
-    QKV buffer, say): the layout the C ABI describes with q_stride_tok / kv_stride_tok."""
-    return (t.dim() == 3 and t.stride(2) == 1 and t.stride(1) == t.shape[2]
-            and t.stride(0) >= t.shape[1] * t.shape[2])
-
-
-def _dev(t, name, dtype=None, token_strided=False):
-    if not t.is_cuda or not (t.is_contiguous() or (token_strided and _token_strided(t))):
-        raise ValueError(f"zipvl: {name} must be a contiguous CUDA tensor" +
-                         (" (or [L, H, d] rows with a token stride)" if token_strided else ""))
-    if dtype is not None and t.dtype != dtype:
+def _dev(t, name, dtype):
+    if not t.is_cuda or not t.is_contiguous():
+        raise ValueError(f"zipvl: {name} must be a contiguous CUDA tensor")
+    if t.dtype != dtype:
         raise TypeError(f"zipvl: {name} must be {dtype}")
     return t
-
-
-def _same_stride(k, v):
-    if k.stride(0) != v.stride(0) or k.shape != v.shape:
-        raise ValueError("zipvl: k and v must have the same shape and token stride")
 
 
 def layer_desc(q, k, softmax_scale=0.0):
@@ -192,16 +198,7 @@ def workspace(nbytes, device):
 def zipvl_score(layer, q, k, probe_pos, acc=None, norm=None, total=None, ws=None, status=None,
                 stream=None):
     """Probe attention scores: returns (acc float32[L], norm float32[L])."""
-    _dev(q, "q", token_strided=True), _dev(k, "k", token_strided=True), _dev(probe_pos, "probe_pos", torch.int32)
-    dev = q.device
-    acc = torch.empty(layer.L, dtype=torch.float32, device=dev) if acc is None else acc
-    norm = torch.empty(layer.L, dtype=torch.float32, device=dev) if norm is None else norm
-    if ws is None:
-        ws = workspace(zipvl_workspace_bytes(OP_SCORE, layer, probe_pos.numel()), dev)
-    _check(load().zipvl_score(C.byref(layer), _ptr(q), _ptr(k), _ptr(probe_pos),
-                              probe_pos.numel(), _ptr(acc), _ptr(norm), _ptr(total), _ptr(ws),
-                              ws.numel(), _ptr(status), _stream(stream)))
-    return acc, norm
+    return (_native or _load_native()).score(layer, q, k, probe_pos, acc, norm, total, ws, status, stream)
 
 
 def keep_last(r: int) -> int:
@@ -212,115 +209,41 @@ def keep_last(r: int) -> int:
 def zipvl_select(acc, norm, tau, mode=0, fixed_k=0, k_out=None, idx=None, kept_mass=None,
                  ws=None, status=None, stream=None):
     """Budget and token set: returns (k_out int32[1], idx int32[L]) on the device."""
-    _dev(acc, "acc", torch.float32), _dev(norm, "norm", torch.float32)
-    L, dev = acc.numel(), acc.device
-    k_out = torch.empty(1, dtype=torch.int32, device=dev) if k_out is None else k_out
-    idx = torch.empty(L, dtype=torch.int32, device=dev) if idx is None else idx
-    if ws is None:
-        lay = zipvl_layer(L, 1, 1, 64, ZIPVL_F32, 0, 0, 0, 0.0, 0)
-        ws = workspace(zipvl_workspace_bytes(OP_SELECT, lay), dev)
-    _check(load().zipvl_select(L, _ptr(acc), _ptr(norm), float(tau), mode, fixed_k, _ptr(k_out),
-                               _ptr(idx), _ptr(kept_mass), _ptr(ws), ws.numel(), _ptr(status),
-                               _stream(stream)))
-    return k_out, idx
+    return (_native or _load_native()).select(acc, norm, tau, mode, fixed_k, k_out, idx, kept_mass, ws, status, stream)
 
 
 def zipvl_sparse_prefill(layer, q, k, v, idx, k_dev, k_max, out=None, out_mode=OUT_PADDED,
                          ws=None, status=None, stream=None):
     """Causal attention over the kept tokens; returns out ([L,Hq,d] or [k_max,Hq,d])."""
-    _dev(q, "q", token_strided=True), _dev(k, "k", token_strided=True), _dev(v, "v", token_strided=True), _dev(idx, "idx", torch.int32)
-    _same_stride(k, v)
-    _dev(k_dev, "k_dev", torch.int32)
-    if out is None:
-        rows = layer.L if out_mode == OUT_PADDED else k_max
-        out = torch.empty((rows, layer.n_q_heads, layer.head_dim), dtype=q.dtype, device=q.device)
-    if ws is None:
-        ws = workspace(zipvl_workspace_bytes(OP_SPARSE_PREFILL, layer), q.device)
-    _check(load().zipvl_sparse_prefill(C.byref(layer), _ptr(q), _ptr(k), _ptr(v), _ptr(idx),
-                                       _ptr(k_dev), int(k_max), _ptr(out), out_mode, _ptr(ws),
-                                       ws.numel(), _ptr(status), _stream(stream)))
-    return out
+    return (_native or _load_native()).sparse_prefill(layer, q, k, v, idx, k_dev, k_max, out, out_mode, ws, status, stream)
 
 
 def zipvl_sparse_prefill_compact(layer, q, k, v, idx, k_dev, k_max, k_cache, v_cache, capacity,
                                  out=None, out_mode=OUT_PADDED, len_out=None, ws=None, status=None,
                                  stream=None):
     """zipvl_sparse_prefill and zipvl_compact_kv in one call; returns (out, len_out)."""
-    _dev(q, "q", token_strided=True), _dev(k, "k", token_strided=True), _dev(v, "v", token_strided=True), _dev(idx, "idx", torch.int32)
-    _same_stride(k, v)
-    _dev(k_dev, "k_dev", torch.int32), _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache")
-    if out is None:
-        rows = layer.L if out_mode == OUT_PADDED else k_max
-        out = torch.empty((rows, layer.n_q_heads, layer.head_dim), dtype=q.dtype, device=q.device)
-    if ws is None:
-        ws = workspace(zipvl_workspace_bytes(OP_SPARSE_PREFILL, layer), q.device)
-    len_out = torch.empty(1, dtype=torch.int32, device=k.device) if len_out is None else len_out
-    _check(load().zipvl_sparse_prefill_compact(
-        C.byref(layer), _ptr(q), _ptr(k), _ptr(v), _ptr(idx), _ptr(k_dev), int(k_max), _ptr(out),
-        out_mode, _ptr(k_cache), _ptr(v_cache), int(capacity), _ptr(len_out), _ptr(ws), ws.numel(),
-        _ptr(status), _stream(stream)))
-    return out, len_out
-
-
-def _batch_desc(q, k):
-    """zipvl_layer + zipvl_batch for stacked Q [n_seq, L, Hq, d] and K [n_seq, L, Hkv, d]
-    (contiguous)."""
-    if q.dim() != 4 or not q.is_contiguous() or not k.is_contiguous():
-        raise ValueError("zipvl: batched calls take contiguous [n_seq, L, H, d] tensors")
-    n_seq, L, Hq, d = q.shape
-    lay = zipvl_layer(L, Hq, k.shape[2], d, _dtype_code(q), 0, 0, 0, 0.0, 0)
-    return lay, zipvl_batch(n_seq, 0, 0, 0)
+    return (_native or _load_native()).sparse_prefill_compact(layer, q, k, v, idx, k_dev, k_max, k_cache, v_cache,
+                                                           capacity, out, out_mode, len_out, ws, status, stream)
 
 
 def zipvl_score_batch(q, k, probe_pos, acc=None, norm=None, ws=None, status=None, stream=None):
     """zipvl_score for stacked sequences: q [n_seq,L,Hq,d], k [n_seq,L,Hkv,d], probe_pos int32
     [n_seq,P]; returns (acc, norm) float32 [n_seq, L]."""
-    _dev(q, "q"), _dev(k, "k"), _dev(probe_pos, "probe_pos", torch.int32)
-    lay, b = _batch_desc(q, k)
-    n_seq, L, P = q.shape[0], q.shape[1], probe_pos.shape[1]
-    acc = torch.empty(n_seq, L, dtype=torch.float32, device=q.device) if acc is None else acc
-    norm = torch.empty(n_seq, L, dtype=torch.float32, device=q.device) if norm is None else norm
-    if ws is None:
-        ws = workspace(load().zipvl_workspace_bytes_batch(OP_SCORE, C.byref(lay), P, n_seq), q.device)
-    _check(load().zipvl_score_batch(C.byref(lay), C.byref(b), _ptr(q), _ptr(k), _ptr(probe_pos), P, _ptr(acc),
-                                    _ptr(norm), None, _ptr(ws), ws.numel(), _ptr(status), _stream(stream)))
-    return acc, norm
+    return (_native or _load_native()).score_batch(q, k, probe_pos, acc, norm, ws, status, stream)
 
 
 def zipvl_select_batch(acc, norm, tau, mode=0, fixed_k=0, k_out=None, idx=None, ws=None, status=None,
                        stream=None):
     """zipvl_select for score rows [n_seq, L]; returns (k_out int32[n_seq], idx int32[n_seq, L])."""
-    _dev(acc, "acc", torch.float32), _dev(norm, "norm", torch.float32)
-    n_seq, L = acc.shape
-    k_out = torch.empty(n_seq, dtype=torch.int32, device=acc.device) if k_out is None else k_out
-    idx = torch.empty(n_seq, L, dtype=torch.int32, device=acc.device) if idx is None else idx
-    if ws is None:
-        lay = zipvl_layer(L, 1, 1, 64, ZIPVL_F32, 0, 0, 0, 0.0, 0)
-        ws = workspace(zipvl_workspace_bytes(OP_SELECT, lay), acc.device)
-    _check(load().zipvl_select_batch(L, n_seq, _ptr(acc), _ptr(norm), float(tau), mode, fixed_k, _ptr(k_out),
-                                     _ptr(idx), None, _ptr(ws), ws.numel(), _ptr(status), _stream(stream)))
-    return k_out, idx
+    return (_native or _load_native()).select_batch(acc, norm, tau, mode, fixed_k, k_out, idx, ws, status, stream)
 
 
 def zipvl_sparse_prefill_batch(q, k, v, idx, k_dev, k_max, k_cache=None, v_cache=None, capacity=0, out=None,
                                out_mode=OUT_PADDED, len_out=None, ws=None, status=None, stream=None):
     """zipvl_sparse_prefill (and, with caches, zipvl_compact_kv) for stacked sequences; returns
     (out [n_seq, L or k_max, Hq, d], len_out or None)."""
-    _dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(idx, "idx", torch.int32), _dev(k_dev, "k_dev", torch.int32)
-    lay, b = _batch_desc(q, k)
-    n_seq, L = q.shape[0], q.shape[1]
-    if out is None:
-        rows = L if out_mode == OUT_PADDED else k_max
-        out = torch.empty((n_seq, rows, lay.n_q_heads, lay.head_dim), dtype=q.dtype, device=q.device)
-    if ws is None:
-        ws = workspace(zipvl_workspace_bytes(OP_SPARSE_PREFILL, lay), q.device)
-    if k_cache is not None and len_out is None:
-        len_out = torch.empty(n_seq, dtype=torch.int32, device=q.device)
-    _check(load().zipvl_sparse_prefill_batch(C.byref(lay), C.byref(b), _ptr(q), _ptr(k), _ptr(v), _ptr(idx),
-                                             _ptr(k_dev), int(k_max), _ptr(out), out_mode, _ptr(k_cache),
-                                             _ptr(v_cache), int(capacity), _ptr(len_out), _ptr(ws), ws.numel(),
-                                             _ptr(status), _stream(stream)))
-    return out, len_out
+    return (_native or _load_native()).sparse_prefill_batch(q, k, v, idx, k_dev, k_max, k_cache, v_cache, capacity, out,
+                                                         out_mode, len_out, ws, status, stream)
 
 
 def zipvl_release_host_scratch():
@@ -333,51 +256,23 @@ def zipvl_release_host_scratch():
 def zipvl_compact_kv(layer, k, v, idx, k_dev, k_max, k_cache, v_cache, capacity, len_out=None,
                      status=None, stream=None):
     """K = K[T], V = V[T] into caller-owned caches; returns len_out int32[1]."""
-    _dev(k, "k", token_strided=True), _dev(v, "v", token_strided=True), _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache")
-    _same_stride(k, v)
-    len_out = torch.empty(1, dtype=torch.int32, device=k.device) if len_out is None else len_out
-    _check(load().zipvl_compact_kv(C.byref(layer), _ptr(k), _ptr(v), _ptr(idx), _ptr(k_dev),
-                                   int(k_max), _ptr(k_cache), _ptr(v_cache), int(capacity),
-                                   _ptr(len_out), _ptr(status), _stream(stream)))
-    return len_out
+    return (_native or _load_native()).compact_kv(layer, k, v, idx, k_dev, k_max, k_cache, v_cache, capacity, len_out,
+                                               status, stream)
 
 
 def zipvl_decode(desc, q, k_new, v_new, k_cache, v_cache, cache_off, capacity, seq_lens, max_len,
                  out=None, ws=None, status=None, stream=None):
     """One decode step over the ragged batch of caches; returns out [B,Hq,d]."""
-    _dev(q, "q"), _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache")
-    _dev(cache_off, "cache_off", torch.int64), _dev(capacity, "capacity", torch.int32)
-    _dev(seq_lens, "seq_lens", torch.int32)
-    out = torch.empty_like(q) if out is None else out
-    if ws is None:
-        lay = zipvl_layer(int(max_len), desc.n_q_heads, desc.n_kv_heads, desc.head_dim, desc.dtype,
-                          0, 0, 0, 0.0, 0)
-        ws = workspace(zipvl_workspace_bytes(OP_DECODE, lay, 0, desc.batch), q.device)
-    _check(load().zipvl_decode(C.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(k_cache),
-                               _ptr(v_cache), _ptr(cache_off), _ptr(capacity), _ptr(seq_lens),
-                               int(max_len), _ptr(out), _ptr(ws), ws.numel(), _ptr(status),
-                               _stream(stream)))
-    return out
+    return (_native or _load_native()).decode(desc, q, k_new, v_new, k_cache, v_cache, cache_off, capacity, seq_lens, max_len,
+                                           out, ws, status, stream)
 
 
 def zipvl_decode_paged(desc, q, k_new, v_new, k_pages, v_pages, block_table, capacity, seq_lens, max_len,
                        out=None, ws=None, status=None, stream=None):
     """One decode step over paged caches: k_pages / v_pages [n_pages, page_rows, Hkv, d],
     block_table int32 [B, max_pages]; returns out [B,Hq,d]."""
-    _dev(q, "q"), _dev(k_pages, "k_pages"), _dev(v_pages, "v_pages")
-    _dev(block_table, "block_table", torch.int32), _dev(capacity, "capacity", torch.int32)
-    _dev(seq_lens, "seq_lens", torch.int32)
-    out = torch.empty_like(q) if out is None else out
-    if ws is None:
-        lay = zipvl_layer(int(max_len), desc.n_q_heads, desc.n_kv_heads, desc.head_dim, desc.dtype,
-                          0, 0, 0, 0.0, 0)
-        ws = workspace(zipvl_workspace_bytes(OP_DECODE, lay, 0, desc.batch), q.device)
-    _check(load().zipvl_decode_paged(C.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(k_pages),
-                                     _ptr(v_pages), _ptr(block_table), block_table.shape[1],
-                                     k_pages.shape[1], k_pages.shape[0], _ptr(capacity), _ptr(seq_lens),
-                                     int(max_len), _ptr(out), _ptr(ws), ws.numel(), _ptr(status),
-                                     _stream(stream)))
-    return out
+    return (_native or _load_native()).decode_paged(desc, q, k_new, v_new, k_pages, v_pages, block_table, capacity, seq_lens,
+                                                 max_len, out, ws, status, stream)
 
 
 class QuantCache:
@@ -405,29 +300,12 @@ class QuantCache:
 
 def zipvl_quantize_kv(layer, k, v, idx, k_dev, k_max, cache, status=None, stream=None):
     """K, V and the token set into the mixed-precision cache; returns cache.lens (device int32[2])."""
-    _dev(k, "k", token_strided=True), _dev(v, "v", token_strided=True), _dev(idx, "idx", torch.int32)
-    _same_stride(k, v)
-    _check(load().zipvl_quantize_kv(C.byref(layer), _ptr(k), _ptr(v), _ptr(idx), _ptr(k_dev), int(k_max),
-                                    _ptr(cache.k_hi), _ptr(cache.v_hi), _ptr(cache.p_hi), cache.cap_hi,
-                                    _ptr(cache.k_lo), _ptr(cache.v_lo), _ptr(cache.p_lo), cache.cap_lo,
-                                    _ptr(cache.lens), _ptr(status), _stream(stream)))
-    return cache.lens
+    return (_native or _load_native()).quantize_kv(layer, k, v, idx, k_dev, k_max, cache, status, stream)
 
 
 def zipvl_decode_quant(desc, q, k_new, v_new, cache, max_len, out=None, ws=None, status=None, stream=None):
     """One decode step of one request over its mixed-precision cache; returns out [1,Hq,d]."""
-    _dev(q, "q")
-    out = torch.empty_like(q) if out is None else out
-    if ws is None:
-        lay = zipvl_layer(int(max_len), desc.n_q_heads, desc.n_kv_heads, desc.head_dim, desc.dtype,
-                          0, 0, 0, 0.0, 0)
-        ws = workspace(zipvl_workspace_bytes(OP_DECODE, lay, 0, 1), q.device)
-    _check(load().zipvl_decode_quant(C.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(cache.k_hi),
-                                     _ptr(cache.v_hi), _ptr(cache.p_hi), cache.cap_hi, _ptr(cache.k_lo),
-                                     _ptr(cache.v_lo), _ptr(cache.p_lo), cache.cap_lo, _ptr(cache.lens),
-                                     int(max_len), _ptr(out), _ptr(ws), ws.numel(), _ptr(status),
-                                     _stream(stream)))
-    return out
+    return (_native or _load_native()).decode_quant(desc, q, k_new, v_new, cache, max_len, out, ws, status, stream)
 
 
 def quant_cache_table(caches, device):
@@ -444,18 +322,7 @@ def quant_cache_table(caches, device):
 def zipvl_decode_quant_batch(desc, q, k_new, v_new, table, max_len, out=None, ws=None, status=None, stream=None):
     """One decode step of desc.batch requests over their mixed-precision caches (table:
     quant_cache_table of the requests' QuantCache objects); returns out [B,Hq,d]."""
-    _dev(q, "q"), _dev(table, "table", torch.int64)
-    if table.shape[0] != desc.batch or table.shape[1] != 8:
-        raise ValueError("table must be int64 [batch, 8]")
-    out = torch.empty_like(q) if out is None else out
-    if ws is None:
-        lay = zipvl_layer(int(max_len), desc.n_q_heads, desc.n_kv_heads, desc.head_dim, desc.dtype,
-                          0, 0, 0, 0.0, 0)
-        ws = workspace(zipvl_workspace_bytes(OP_DECODE, lay, 0, desc.batch), q.device)
-    _check(load().zipvl_decode_quant_batch(C.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(table),
-                                           int(max_len), _ptr(out), _ptr(ws), ws.numel(), _ptr(status),
-                                           _stream(stream)))
-    return out
+    return (_native or _load_native()).decode_quant_batch(desc, q, k_new, v_new, table, max_len, out, ws, status, stream)
 
 
 def zipvl_decode_noalloc(desc, q, k_new, v_new, k_cache, v_cache, cache_off, capacity, seq_lens,
@@ -463,14 +330,8 @@ def zipvl_decode_noalloc(desc, q, k_new, v_new, k_cache, v_cache, cache_off, cap
     """zipvl_decode for callers that cannot allocate: the scratch is a fixed
     array inside the library, and this wrapper allocates nothing either (the
     caller passes `out`).  Raises ZipvlError (workspace) beyond the 8 MiB limit."""
-    _dev(q, "q"), _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache"), _dev(out, "out")
-    _dev(cache_off, "cache_off", torch.int64), _dev(capacity, "capacity", torch.int32)
-    _dev(seq_lens, "seq_lens", torch.int32)
-    _check(load().zipvl_decode_noalloc(C.byref(desc), _ptr(q), _ptr(k_new), _ptr(v_new),
-                                       _ptr(k_cache), _ptr(v_cache), _ptr(cache_off),
-                                       _ptr(capacity), _ptr(seq_lens), int(max_len), _ptr(out),
-                                       _ptr(status), _stream(stream)))
-    return out
+    return (_native or _load_native()).decode_noalloc(desc, q, k_new, v_new, k_cache, v_cache, cache_off, capacity,
+                                                   seq_lens, max_len, out, status, stream)
 
 
 def zipvl_selftest_wait_timeout(poll_limit, progress, status, stream=None):
