@@ -164,8 +164,8 @@ zipvl_status zipvl_sparse_prefill(const zipvl_layer *layer, const void *q, const
         return launch_prefill_tc(a, q, k, v, idx, k_dev, k_max, out, out_mode, nullptr, nullptr, 0, nullptr,
                                  ws, status_word, st);
     }
-    return launch_prefill_simt(a, layer->dtype, q, k, v, idx, k_dev, k_max, out, out_mode,
-                               status_word, st);
+    return launch_prefill_simt(a, layer->dtype, q, k, v, idx, k_dev, k_max, out, out_mode, nullptr, nullptr, 0,
+                               nullptr, status_word, st);
 }
 
 zipvl_status zipvl_sparse_prefill_compact(const zipvl_layer *layer, const void *q, const void *k,
@@ -196,9 +196,11 @@ zipvl_status zipvl_sparse_prefill_compact(const zipvl_layer *layer, const void *
         return launch_prefill_tc(a, q, k, v, idx, k_dev, k_max, out, out_mode, k_cache, v_cache, capacity,
                                  len_out, ws, status_word, st);
     }
-    // other shapes and types: the two kernels one after the other
-    s = launch_prefill_simt(a, layer->dtype, q, k, v, idx, k_dev, k_max, out, out_mode, status_word, st);
-    if (s != ZIPVL_OK) return s;
+    // fp32: one kernel as well; other shapes of 16-bit storage: the two kernels one after the other
+    const bool one = layer->dtype == ZIPVL_F32;
+    s = launch_prefill_simt(a, layer->dtype, q, k, v, idx, k_dev, k_max, out, out_mode, one ? k_cache : nullptr,
+                            one ? v_cache : nullptr, capacity, len_out, status_word, st);
+    if (s != ZIPVL_OK || one) return s;
     return launch_compact(a, elem_bytes(layer->dtype), k, v, idx, k_dev, k_max, k_cache,
                           v_cache, capacity, len_out, status_word, st);
 }

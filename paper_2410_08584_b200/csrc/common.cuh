@@ -111,6 +111,27 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The same with thread-block clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           unsigned int cluster, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // ---- launchers implemented per file -----------------------------------------
 struct LayerArgs {
     int L, Hq, Hkv, D, G;
@@ -135,8 +156,9 @@ size_t select_ws_bytes();
 
 zipvl_status launch_prefill_simt(const LayerArgs &a, int dtype, const void *q, const void *k,
                                  const void *v, const int32_t *idx, const int32_t *k_dev,
-                                 int k_max, void *out, int out_mode, int32_t *status_word,
-                                 cudaStream_t st);
+                                 int k_max, void *out, int out_mode, void *kc, void *vc, int capacity,
+                                 int32_t *len_out, int32_t *status_word, cudaStream_t st);
+// (kc == nullptr: attention only; otherwise fp32 tensors are compacted too)
 
 zipvl_status launch_compact(const LayerArgs &a, int elem_bytes, const void *k, const void *v,
                             const int32_t *idx, const int32_t *k_dev, int k_max, void *k_cache,
