@@ -10,7 +10,17 @@
 //           column sum of exp2(s - m_r) / l_r over the probes that see the key;
 //   pass 3  sum over heads in fixed order, nnz by binary search, normalise.
 // Nothing uses float atomics, so results repeat bit for bit.
+//
+// Short fp32 layers (kClusterKeys x 8 keys, 128 probes) take one sweep instead of two: a cluster of
+// eight CTAs holds the scores of 32 probes against all keys of a head in registers, exchanges the row
+// statistics through distributed shared memory and adds up the columns from the exponentials
+// it already has.  The 1024-token, 4-head layer is 34 MFLOP of scores: what counts is the number
+// of SMs at work (64 instead of 16) and the length of a thread's chain (2 x 4 register tiles over
+// 128 keys instead of a dot product per key): 56 -> 11 us with the sum over heads.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace zipvl {
 namespace {
@@ -182,6 +192,153 @@ score_colsum_kernel(LayerArgs a, const T *__restrict__ q, const T *__restrict__ 
     if (j < a.L) partial[(long long)h * a.L + j] = colsum;
 }
 
+constexpr int kClThreads = 256, kClProbes = 32, kClTile = 64;
+constexpr int kClusterKeys = 4 * kClTile;   // keys a CTA can hold: 4 tiles x 8 scores in registers per thread
+
+// grid (8 CTAs of a cluster, head, tile of 32 probes); NS = 64-key tiles per CTA.
+// A thread owns rows row0 + 2 i (i < 2) and keys tx + 16 j (j < 4) of every tile; rows are padded by
+// 16 bytes so that the float4 reads of a warp (2 rows, 16 keys) are conflict-free, and lanes 2i, 2i + 1
+// share their keys (pairs of equal addresses make a 16-byte read two cycles instead of four).
+template <int D, int NS>
+__global__ void __launch_bounds__(kClThreads)
+score_cluster_kernel(LayerArgs a, const float *__restrict__ q, const float *__restrict__ k,
+                     const int32_t *__restrict__ probe_pos, int P, int keys_per_cta, float *__restrict__ partial,
+                     int32_t *status_word) {
+    constexpr int QP = D + 4, CH = D / 4;
+    extern __shared__ __align__(16) float smem[];
+    float *Qs = smem;                                   // [32][QP]
+    float *Ks = Qs + kClProbes * QP;                    // two tiles [64][QP]
+    float *part = Ks + 2 * kClTile * QP;                // column sums [8 warps][NS * 64]
+    float *weight = part + 8 * NS * kClTile;            // [32]
+    float2 *stat = reinterpret_cast<float2 *>(weight + kClProbes);   // [32] this CTA's (m, l)
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+
+    grid_launch_dependents();
+    grid_dependency_wait(q, k, probe_pos);
+    const int rank = blockIdx.x, h = blockIdx.y, z = blockIdx.z, g = h / a.G;
+    const int tid = threadIdx.x, tx = (tid & 31) >> 1, warp = tid >> 5;
+    const int row0 = warp * 4 + (tid & 1);
+    const int j0 = rank * keys_per_cta, j1 = min(a.L, j0 + keys_per_cta);
+
+    auto load_keys = [&](int t) {
+        float *dst = Ks + (t & 1) * kClTile * QP;
+        for (int e = tid; e < kClTile * CH; e += kClThreads) {
+            const int r = e / CH, c = (e % CH) * 4, j = j0 + t * kClTile + r;
+            ptx::cp_async16(ptx::smem_u32(dst + r * QP + c), k + (long long)(j < j1 ? j : 0) * a.kv_stride + (long long)g * D + c,
+                            j < j1 ? 16u : 0u);
+        }
+        ptx::cp_async_commit();
+    };
+    auto position = [&](int r) {                        // of probe r of this tile; -1: none or out of range
+        const int p = z * kClProbes + r;
+        const int c = p < P ? probe_pos[p] : -1;
+        return c < a.L ? c : -1;
+    };
+    for (int e = tid; e < kClProbes * CH; e += kClThreads) {
+        const int r = e / CH, c = (e % CH) * 4, pos = position(r);
+        if (pos < 0 && c == 0 && h == 0 && rank == 0 && z * kClProbes + r < P) report(status_word, ZIPVL_DEV_BAD_INDEX);
+        ptx::cp_async16(ptx::smem_u32(Qs + r * QP + c), q + (long long)max(pos, 0) * a.q_stride + (long long)h * D + c,
+                        pos >= 0 ? 16u : 0u);
+    }
+    load_keys(0);
+    if (NS > 1) load_keys(1);
+    const int pos[2] = {position(row0), position(row0 + 2)};
+
+    float s[NS][2][4];
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+        if (t + 1 < NS) ptx::cp_async_wait<1>(); else ptx::cp_async_wait<0>();
+        __syncthreads();
+        const float *kt = Ks + (t & 1) * kClTile * QP;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[t][i][j] = 0.f;
+#pragma unroll 4
+        for (int c = 0; c < CH; ++c) {
+            float4 x[2], y[4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) x[i] = *reinterpret_cast<const float4 *>(Qs + (row0 + 2 * i) * QP + 4 * c);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4 *>(kt + (tx + 16 * j) * QP + 4 * c);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    s[t][i][j] = fmaf(x[i].x, y[j].x, s[t][i][j]);
+                    s[t][i][j] = fmaf(x[i].y, y[j].y, s[t][i][j]);
+                    s[t][i][j] = fmaf(x[i].z, y[j].z, s[t][i][j]);
+                    s[t][i][j] = fmaf(x[i].w, y[j].w, s[t][i][j]);
+                }
+        }
+        if (t + 2 < NS) {
+            __syncthreads();
+            load_keys(t + 2);
+        }
+    }
+    // row statistics over this CTA's keys; s becomes exp2(s - m)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        float m = -INFINITY;
+#pragma unroll
+        for (int t = 0; t < NS; ++t)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int key = j0 + t * kClTile + tx + 16 * j;
+                s[t][i][j] = (key < j1 && key <= pos[i]) ? s[t][i][j] * a.scale_log2 : -INFINITY;
+                m = fmaxf(m, s[t][i][j]);
+            }
+#pragma unroll
+        for (int off = 16; off > 1; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        const float ref = m == -INFINITY ? 0.f : m;
+        float l = 0.f;
+#pragma unroll
+        for (int t = 0; t < NS; ++t)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                s[t][i][j] = fast_exp2(s[t][i][j] - ref);
+                l += s[t][i][j];
+            }
+#pragma unroll
+        for (int off = 16; off > 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+        if (tx == 0) stat[row0 + 2 * i] = make_float2(m, l);
+    }
+    cl.sync();
+    if (tid < kClProbes) {                              // what this CTA's exponentials of row tid count for
+        float2 st[8];
+        float M = -INFINITY, sum = 0.f;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            st[p] = *(cl.map_shared_rank(stat, p) + tid);
+            M = fmaxf(M, st[p].x);
+        }
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            if (st[p].y > 0.f) sum += st[p].y * fast_exp2(st[p].x - M);
+        const float2 own = stat[tid];
+        weight[tid] = own.y > 0.f ? fast_exp2(own.x - M) / sum : 0.f;
+    }
+    cl.sync();                                          // (also: nobody leaves while its statistics are read)
+    const float w0 = weight[row0], w1 = weight[row0 + 2];
+#pragma unroll
+    for (int t = 0; t < NS; ++t)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float v = s[t][0][j] * w0 + s[t][1][j] * w1;
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            if (!(tid & 1)) part[warp * NS * kClTile + t * kClTile + tx + 16 * j] = v;
+        }
+    __syncthreads();
+    for (int e = tid; e < NS * kClTile; e += kClThreads) {
+        if (j0 + e >= j1) break;
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += part[w * NS * kClTile + e];
+        partial[((long long)h * gridDim.z + z) * a.L + j0 + e] = v;
+    }
+}
+
 // first r with probe_pos[r] >= x (probe_pos ascending)
 __device__ __forceinline__ int lower_bound(const int32_t *p, int n, int x) {
     int lo = 0, hi = n;
@@ -192,13 +349,17 @@ __device__ __forceinline__ int lower_bound(const int32_t *p, int n, int x) {
     return lo;
 }
 
-__global__ void score_finalize_kernel(int L, int Hq, int P, const float *__restrict__ partial,
+// n_part: partial rows to add up, in order (heads, or heads x probe tiles)
+__global__ void score_finalize_kernel(int L, int Hq, int n_part, int P, const float *__restrict__ partial,
                                       const int32_t *__restrict__ probe_pos,
                                       float *__restrict__ acc, float *__restrict__ norm) {
+    grid_launch_dependents();
+    grid_dependency_wait(partial, probe_pos);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= L) return;
     float s = 0.f;
-    for (int h = 0; h < Hq; ++h) s += partial[(long long)h * L + j];
+#pragma unroll 8
+    for (int h = 0; h < n_part; ++h) s += partial[(long long)h * L + j];
     // structural nnz: probes at positions j .. L-1
     const int nnz = lower_bound(probe_pos, P, L) - lower_bound(probe_pos, P, j);
     acc[j] = s;
@@ -220,11 +381,44 @@ __global__ void sum_to_double_kernel(int L, const float *__restrict__ x, double 
     if (threadIdx.x == 0) *out = sh[0];
 }
 
+static bool use_cluster(int L, int P) { return L <= 8 * kClusterKeys && P <= 128; }
+
 size_t score_simt_ws_bytes(int L, int Hq, int P) {
     const size_t n_chunks = (L + kChunk - 1) / kChunk;
     size_t stats = (size_t)Hq * n_chunks * P * sizeof(float2);
     stats = (stats + 255) & ~(size_t)255;
-    return stats + (size_t)Hq * L * sizeof(float);
+    const size_t cluster = (size_t)Hq * ((P + kClProbes - 1) / kClProbes) * L * sizeof(float);
+    const size_t two_pass = stats + (size_t)Hq * L * sizeof(float);
+    return use_cluster(L, P) && cluster > two_pass ? cluster : two_pass;
+}
+
+template <int D, int NS>
+static zipvl_status run_cluster(const LayerArgs &a, const float *q, const float *k, const int32_t *probe_pos, int P,
+                                float *acc, float *norm, double *total, float *partial, int32_t *status_word,
+                                cudaStream_t st) {
+    const size_t smem = sizeof(float) * ((kClProbes + 2 * kClTile) * (D + 4) + 8 * NS * kClTile + 3 * kClProbes);
+    cudaError_t e = cudaFuncSetAttribute(score_cluster_kernel<D, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "score: smem opt-in: %s", cudaGetErrorString(e));
+    const int nz = (P + kClProbes - 1) / kClProbes;
+    e = launch_cluster(score_cluster_kernel<D, NS>, dim3(8, a.Hq, nz), dim3(kClThreads), smem, st, 8, a, q, k, probe_pos, P,
+                       (a.L + 7) / 8, partial, status_word);
+    if (e == cudaSuccess)
+        e = launch_dependent(score_finalize_kernel, dim3((a.L + 63) / 64), dim3(64), 0, st, a.L, a.Hq, a.Hq * nz, P,
+                             partial, probe_pos, acc, norm);
+    if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "score: launch: %s", cudaGetErrorString(e));
+    if (total) sum_to_double_kernel<<<1, 1024, 0, st>>>(a.L, acc, total);
+    count_launches(total ? 3 : 2);
+    return check_launch("zipvl_score");
+}
+
+template <int D>
+static zipvl_status run_cluster(const LayerArgs &a, const float *q, const float *k, const int32_t *probe_pos, int P,
+                                float *acc, float *norm, double *total, float *partial, int32_t *status_word,
+                                cudaStream_t st) {
+    const int keys = (a.L + 7) / 8;
+    if (keys <= kClTile) return run_cluster<D, 1>(a, q, k, probe_pos, P, acc, norm, total, partial, status_word, st);
+    if (keys <= 2 * kClTile) return run_cluster<D, 2>(a, q, k, probe_pos, P, acc, norm, total, partial, status_word, st);
+    return run_cluster<D, 4>(a, q, k, probe_pos, P, acc, norm, total, partial, status_word, st);
 }
 
 template <typename T, int D>
@@ -249,7 +443,7 @@ static zipvl_status run(const LayerArgs &a, const void *q, const void *k,
     dim3 g2((a.L + kThreads - 1) / kThreads, a.Hq);
     score_colsum_kernel<T, D><<<g2, kThreads, smem, st>>>(a, (const T *)q, (const T *)k, probe_pos,
                                                          P, n_chunks, stats, partial);
-    score_finalize_kernel<<<(a.L + 255) / 256, 256, 0, st>>>(a.L, a.Hq, P, partial, probe_pos, acc,
+    score_finalize_kernel<<<(a.L + 255) / 256, 256, 0, st>>>(a.L, a.Hq, a.Hq, P, partial, probe_pos, acc,
                                                             norm);
     if (total) sum_to_double_kernel<<<1, 1024, 0, st>>>(a.L, acc, total);
     count_launches(total ? 4 : 3);
@@ -260,6 +454,12 @@ zipvl_status launch_score_simt(const LayerArgs &a, int dtype, const void *q, con
                                const int32_t *probe_pos, int P, float *acc, float *norm,
                                double *total, void *ws, int32_t *status_word, cudaStream_t st) {
     if (P > 8192) return fail(ZIPVL_ERR_UNSUPPORTED, "score: n_probe %d > 8192", P);
+    if (dtype == ZIPVL_F32 && use_cluster(a.L, P)) {
+        // one sweep: every (head, 32 probes) is one cluster whose scores fit the registers of its CTAs
+        auto *one = a.D == 64 ? run_cluster<64> : a.D == 96 ? run_cluster<96> : a.D == 128 ? run_cluster<128> : nullptr;
+        if (one)
+            return one(a, (const float *)q, (const float *)k, probe_pos, P, acc, norm, total, (float *)ws, status_word, st);
+    }
     if (dtype == ZIPVL_F32) {
         if (a.D == 64) return run<float, 64>(a, q, k, probe_pos, P, acc, norm, total, ws, status_word, st);
         if (a.D == 96) return run<float, 96>(a, q, k, probe_pos, P, acc, norm, total, ws, status_word, st);
