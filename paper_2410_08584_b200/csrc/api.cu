@@ -2,6 +2,8 @@
 // No kernel lives here.  Every entry point validates on the host, launches on
 // the caller's stream and returns without synchronising.
 #include <math.h>
+
+#include <algorithm>
 #include <mutex>
 #include <stdarg.h>
 #include <stdio.h>
@@ -97,7 +99,9 @@ size_t zipvl_workspace_bytes(int32_t op, const zipvl_layer *layer, int32_t n_pro
         case ZIPVL_OP_COMPACT_KV: return 256;
         case ZIPVL_OP_DECODE:
             if (batch < 1) return 0;
-            return align256(decode_ws_bytes(batch, a.Hq, a.D, a.L, a.Hkv, layer->dtype));
+            // (the decode over a mixed-precision cache takes its workspace by the same query)
+            return align256(std::max(decode_ws_bytes(batch, a.Hq, a.D, a.L, a.Hkv, layer->dtype),
+                                     decode_quant_ws_bytes(batch, a.Hq, a.Hkv, a.D, a.L)));
     }
     return 0;
 }

@@ -175,12 +175,14 @@ struct PageArgs {
 // (Hkv and dtype decide whether the grouped-query tensor-core kernel, which leaves more partials,
 // may run: 0 / -1 = the CUDA-core layout)
 size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv = 0, int dtype = -1);
-int decode_chunk_rows(int B, int Hq, int max_len);
-size_t decode_partial_bytes(int B, int Hq, int D, int max_len);
+// workspace of the decode over the mixed-precision cache (kvquant_decode.cu)
+size_t decode_quant_ws_bytes(int B, int Hq, int Hkv, int D, int max_len);
+// caches != nullptr: the new length of request b goes to caches[b].lens[0] instead of seq_lens[b];
 // used != nullptr: used[b * (Hq / group) + hq / group] of the n_chunks slots hold a partial
 zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int chunk, int n_chunks, const float *ws,
                                  const int *lens, int32_t *seq_lens, void *out, cudaStream_t st,
-                                 const int *used = nullptr, int group = 1);
+                                 const int *used = nullptr, int group = 1,
+                                 const zipvl_quant_cache *caches = nullptr);
 // Grouped-query decode on the tensor cores: 16-bit storage, head_dim 64 / 96 / 128, 2 to 32 query
 // heads per kv head.  Two kernels that leave partials in the layout of the kernels in decode.cu and the
 // (length, appended) pairs in lens[]; the caller launches the merge.

@@ -288,10 +288,10 @@ template <typename T, int D, int kMergeUnroll>
 __global__ void __launch_bounds__(256, kMergeUnroll == 8 ? 4 : 5)
 decode_merge_kernel(int Hq, int lanes, int n_chunks, const float *__restrict__ ws,
                     const int *__restrict__ lens, int32_t *__restrict__ seq_lens, T *__restrict__ out,
-                    const int *__restrict__ used, int group) {
+                    const int *__restrict__ used, int group, const zipvl_quant_cache *__restrict__ caches) {
     static_assert(D % 2 == 0, "two channels per thread");
     grid_launch_dependents();
-    grid_dependency_wait(ws, lens, seq_lens, used);
+    grid_dependency_wait(ws, lens, seq_lens, used, caches);
     const int b = blockIdx.y;
     const int t = (blockIdx.x * 256 + threadIdx.x) / lanes;             // (head, channel pair) of this lane group
     const int part = threadIdx.x % lanes;
@@ -342,7 +342,7 @@ decode_merge_kernel(int Hq, int lanes, int n_chunks, const float *__restrict__ w
     if (live && part == 0)
         store2(out + ((long long)b * Hq + hq) * D + c, Ls > 0.f ? O0 / Ls : 0.f, Ls > 0.f ? O1 / Ls : 0.f);
     // Eq. 4: the appended row now counts
-    if (blockIdx.x == 0 && threadIdx.x == 0 && lens[2 * b + 1]) seq_lens[b] = lens[2 * b];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && lens[2 * b + 1]) *(caches ? caches[b].lens : seq_lens + b) = lens[2 * b];
 }
 
 // Lanes per (head, channel pair) of the merge: as many as there are slots to share (at most
@@ -421,7 +421,7 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
         const int lanes = merge_lanes(B, Hq, D, n_chunks);
         le = launch_dependent(decode_merge_kernel<T, D, 8>, merge_grid(B, Hq, D, lanes), dim3(256), 0, st, Hq,
                               lanes, n_chunks, (const float *)wsf, (const int *)lens, seq_lens, (T *)out,
-                              (const int *)nullptr, 1);
+                              (const int *)nullptr, 1, (const zipvl_quant_cache *)nullptr);
     }
     if (le != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "zipvl_decode: launch: %s", cudaGetErrorString(le));
     count_launches(2);
@@ -430,19 +430,17 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
 
 }  // namespace
 
-// what the decode over a quantised cache (kvquant.cu) shares with this file: the chunking, the
-// layout of the partial results and the merge kernel
-int decode_chunk_rows(int B, int Hq, int max_len) { return decode_chunk(B, Hq, max_len); }
-size_t decode_partial_bytes(int B, int Hq, int D, int max_len) { return partial_bytes(B, Hq, D, max_len); }
+// what the tensor-core kernels and the decode over a quantised cache (kvquant_decode.cu) share with
+// this file: the layout of the partial results and the merge kernel
 zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int chunk, int n_chunks, const float *ws,
                                  const int *lens, int32_t *seq_lens, void *out, cudaStream_t st,
-                                 const int *used, int group) {
+                                 const int *used, int group, const zipvl_quant_cache *caches) {
     cudaError_t le = cudaErrorInvalidValue;
     (void)chunk;
     const int lanes = merge_lanes(B, Hq, D, n_chunks);
     const dim3 grid = merge_grid(B, Hq, D, lanes);
 #define ZIPVL_MERGE(T_, D_) \
-    le = launch_dependent(decode_merge_kernel<T_, D_, 6>, grid, dim3(256), 0, st, Hq, lanes, n_chunks, ws, lens, seq_lens, (T_ *)out, used, group)
+    le = launch_dependent(decode_merge_kernel<T_, D_, 6>, grid, dim3(256), 0, st, Hq, lanes, n_chunks, ws, lens, seq_lens, (T_ *)out, used, group, caches)
     if (dtype == ZIPVL_BF16 && D == 128) ZIPVL_MERGE(__nv_bfloat16, 128);
     else if (dtype == ZIPVL_BF16 && D == 96) ZIPVL_MERGE(__nv_bfloat16, 96);
     else if (dtype == ZIPVL_BF16 && D == 64) ZIPVL_MERGE(__nv_bfloat16, 64);

@@ -167,3 +167,39 @@ def test_batched_decode_over_quantised_caches(zipvl, case):
     for b in (0, 2, 3):
         assert torch.equal(out[b], good[b])
     assert [c.lens.tolist() for c in caches] == before
+
+
+@pytest.mark.parametrize("n_hi,n_lo,Hq,Hkv,d,dtype", [
+    (1, 0, 1, 1, 64, torch.bfloat16), (31, 1, 5, 5, 128, torch.float16), (32, 33, 8, 2, 128, torch.bfloat16),
+    (63, 500, 4, 2, 64, torch.float16), (0, 65, 2, 2, 128, torch.bfloat16), (700, 129, 16, 4, 64, torch.bfloat16)])
+@pytest.mark.parametrize("spread", [1.0, 1e4])
+def test_quantised_decode_at_the_edges_of_its_steps(zipvl, n_hi, n_lo, Hq, Hkv, d, dtype, spread):
+    """Rows around the 32-row steps and the boundary between the blocks, kv heads that do not fill a CTA, values
+    whose scales span several orders of magnitude (spread), an appended row that opens a step."""
+    z = zipvl
+    storage, code = ("f16", z.ZIPVL_F16) if dtype == torch.float16 else ("bf16", z.ZIPVL_BF16)
+    L = n_hi + n_lo
+    g = torch.Generator().manual_seed(L + Hq)
+    k, v = torch.randn(L, Hkv, d, generator=g), torch.randn(L, Hkv, d, generator=g)
+    if spread > 1:
+        v *= torch.exp(torch.rand(L, Hkv, 1, generator=g) * np.log(spread)) / spread
+    k, v = k.to(dtype), v.to(dtype)
+    T = torch.sort(torch.randperm(L, generator=g)[:n_hi]).values
+    idx = torch.full((L,), -1, dtype=torch.int32)
+    idx[:n_hi] = T.to(torch.int32)
+    cache = z.QuantCache(L, Hkv, d, dtype, DEV, cap_hi=n_hi + 2, cap_lo=n_lo + 1)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    z.zipvl_quantize_kv(z.layer_desc(k, k), k.to(DEV), v.to(DEV), idx.to(DEV),
+                        torch.tensor([n_hi], dtype=torch.int32, device=DEV), L, cache, status=st)
+    ref = oracle.quantize_kv(to_np(k), to_np(v), T.numpy(), storage)
+    desc = z.zipvl_decode_desc(1, Hq, Hkv, d, code, 0.0)
+    for _ in range(2):
+        q = torch.randn(1, Hq, d, generator=g).to(dtype)
+        kn, vn = (torch.randn(1, Hkv, d, generator=g).to(dtype) / (1 if i == 0 else spread) for i in range(2))
+        out = z.zipvl_decode_quant(desc, q.to(DEV), kn.to(DEV), vn.to(DEV), cache, L + 2, status=st)
+        want = oracle.decode_step_quant(to_np(q), to_np(kn), to_np(vn), ref, Hkv, storage)
+        scale = np.abs(want).max()
+        err = np.abs(to_np(out) - want).max() / scale
+        assert err < (2e-3 if storage == "f16" else 8e-3), err
+    assert st.item() == 0 and cache.lens.tolist() == [n_hi + 2, n_lo]
+    _check_blocks(_blocks_from_gpu(cache, n_hi + 2, n_lo), ref)
