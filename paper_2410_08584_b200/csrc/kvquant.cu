@@ -21,83 +21,215 @@ namespace {
 
 using namespace kvq;
 
-constexpr int kQuantThreads = 256;
-constexpr int kQuantIters = 8;      // (token, head) pairs per lane group and CTA
+// What bounds the encoder: it reads 4 bytes and writes about 1 per (channel of K and V), so HBM has
+// to be kept busy at some 25 values per SM and cycle, i.e. with about ten instructions per value at
+// most.  One lane per eight channels, a division and a reciprocal per lane and tensor, a
+// conversion each way per value and, in front of all, a 12-step binary search per token took 30 us for
+// the 2944-token, 32-head layer (60 MB).  Here
+//   - eight lanes share a row of 64 or 128 channels of K and V of two (token, head) pairs, so the four
+//     divisions and reciprocals of a group are done by four different lanes at once;
+//   - the row's maximum and negated minimum travel in one register of packed 16-bit values (the
+//     minimum is an element: storing it as the row's zero rounds nothing);
+//   - rint is an addition of 1.5 * 2^23 (exact to even for the values up to 15 that occur), and the
+//     sums of the code words' terms come out by integer multiply-adds modulo 2^32;
+//   - the loads of a CTA's first rows are under way while the token set is searched, 32 ways at a time.
+// 30 -> 17 us.
+constexpr int kQuantThreads = 128;
+constexpr int kQuantIters = 4;      // steps of 32 (token, head) pairs per CTA
+constexpr int kQuantPairs = (kQuantThreads / 8) * 2;
+
+// packed pair of storage-type values
+template <bool kHalf>
+__device__ __forceinline__ uint32_t pk_max(uint32_t a, uint32_t b) {        // NaN if either is
+    uint32_t d;
+    if (kHalf) asm("max.NaN.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    else asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+template <bool kHalf>
+__device__ __forceinline__ uint32_t pk_min(uint32_t a, uint32_t b) {
+    uint32_t d;
+    if (kHalf) asm("min.NaN.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    else asm("min.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
 
 template <bool kHalf, int D>
-__global__ void __launch_bounds__(kQuantThreads)
+__global__ void __launch_bounds__(kQuantThreads, 5)
 quantize_kv_kernel(LayerArgs a, const unsigned short *__restrict__ k, const unsigned short *__restrict__ v,
                    const int32_t *__restrict__ idx, const int32_t *__restrict__ k_dev, int k_max,
                    QuantBlocks qb, int32_t *__restrict__ lens_out, int32_t *status_word) {
-    constexpr int kLanes = D / 8;                 // lanes per (token, head)
-    constexpr int kGroups = 32 / kLanes;          // groups per warp
+    constexpr int P = D / 64;                     // 16-byte pieces per lane (8 lanes to a row)
+    constexpr int kPairsPerCta = kQuantPairs * kQuantIters;
+    __shared__ int s_row[kPairsPerCta + 2];       // where a token goes: >= 0: hi row; < 0: -(lo row) - 1
+    __shared__ int s_entry[kPairsPerCta + 2], s_low;
     grid_launch_dependents();
     grid_dependency_wait(k, v, idx, k_dev);       // T and k are the selection's output
+    const int lane = threadIdx.x & 31, lg = lane & 7;
+    // (pair numbers fit 32 bits: 2^32 rows of K alone would be half a terabyte)
+    const uint32_t n_pairs = (uint32_t)a.L * (uint32_t)a.Hkv, p0 = blockIdx.x * (uint32_t)kPairsPerCta;
+    const uint32_t t_first = p0 / (uint32_t)a.Hkv, g_first = p0 - t_first * (uint32_t)a.Hkv;
+    const unsigned long long inv_heads = ((1ull << 32) + a.Hkv - 1) / (uint32_t)a.Hkv;    // exact quotients below 2^16
+    // combination u: tensor u & 1 (K, V) of pair u >> 1 of this group of lanes
+    uint4 w[4][P];
+    auto pair_of = [&](int it, int half) { return p0 + (uint32_t)(it * kQuantPairs + (threadIdx.x >> 3) * 2 + half); };
+    auto token_of = [&](uint32_t p) { return (uint32_t)(((unsigned long long)(p - p0 + g_first) * inv_heads) >> 32); };   // behind t_first
+    auto load = [&](int it) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t p = pair_of(it, half);
+            if (p < n_pairs) {
+                const uint32_t j = token_of(p), h = p - p0 + g_first - j * (uint32_t)a.Hkv;
+                const long long off = (long long)(t_first + j) * a.kv_stride + h * D + lg * 8;
+#pragma unroll
+                for (int i = 0; i < P; ++i) {
+                    w[2 * half][i] = __ldg(reinterpret_cast<const uint4 *>(k + off + i * 64));
+                    w[2 * half + 1][i] = __ldg(reinterpret_cast<const uint4 *>(v + off + i * 64));
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < P; ++i) { w[2 * half][i] = make_uint4(0, 0, 0, 0); w[2 * half + 1][i] = make_uint4(0, 0, 0, 0); }
+            }
+        }
+    };
+    load(0);
     int n = *k_dev;
     if (n > k_max || n < 0) {
         if (blockIdx.x == 0 && threadIdx.x == 0) report(status_word, ZIPVL_DEV_CAPACITY);
         n = n < 0 ? 0 : k_max;
     }
-    if (n > qb.cap_hi || a.L - n > qb.cap_lo) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) report(status_word, ZIPVL_DEV_CAPACITY);
-    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (n > qb.cap_hi || a.L - n > qb.cap_lo) report(status_word, ZIPVL_DEV_CAPACITY);
         lens_out[0] = min(n, qb.cap_hi);
         lens_out[1] = min(a.L - n, qb.cap_lo);
     }
-    // A CTA takes kPairsPerCta consecutive (token, head) pairs, i.e. a short run of tokens.
-    // Where each of those tokens goes -- row i of the 4-bit block if it is T's i-th entry, else
-    // row (t - #entries of T below t) of the 2-bit block -- is looked up once per token (a
-    // binary search in the ascending list) by the first threads and shared.
-    constexpr int kPairsPerIter = (kQuantThreads / 32) * kGroups;
-    constexpr int kPairsPerCta = kPairsPerIter * kQuantIters;
-    __shared__ int s_row[kPairsPerCta + 2];            // >= 0: hi row; < 0: -(lo row) - 1
-    const int lane = threadIdx.x & 31, lg = lane % kLanes;
-    const long long n_pairs = (long long)a.L * a.Hkv;
-    const long long p0 = (long long)blockIdx.x * kPairsPerCta;
-    const int t_first = (int)(p0 / a.Hkv);
-    const int t_last = (int)(min(p0 + kPairsPerCta, n_pairs) - 1) / a.Hkv;
-    for (int t = t_first + (int)threadIdx.x; t <= t_last; t += kQuantThreads) {
-        int lo = 0, hi = n;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (idx[mid] < t) lo = mid + 1; else hi = mid;
+    // A CTA takes consecutive (token, head) pairs, i.e. a short run of tokens.  Where each of those
+    // goes -- row i of the 4-bit block if it is T's i-th entry, else row (t - #entries of T below t)
+    // of the 2-bit block -- is looked up once: the first warp finds the first entry >= t_first,
+    // splitting the range 32 ways per step, and the entries behind it are compared.
+    const int count = (int)token_of(min(p0 + kPairsPerCta, n_pairs) - 1) + 1;
+    if (threadIdx.x < 32) {
+        const int tf = (int)t_first;
+        int lo = max(0, tf - (a.L - n)), hi = max(lo, min(n, tf));   // (ascending: idx[i] >= i, and L - n are left out)
+        while (lo < hi) {                         // idx[lo - 1] < t_first <= idx[hi]
+            const int step = (hi - lo + 31) / 32, at = lo + (lane + 1) * step - 1;
+            const bool below = at < hi && idx[at] < tf;
+            const int c = __popc(__ballot_sync(0xffffffffu, below));
+            lo += c * step;
+            hi = min(hi, lo + step - 1);
         }
-        s_row[t - t_first] = (lo < n && idx[lo] == t) ? lo : -(t - lo) - 1;
+        if (lane == 0) s_low = lo;
     }
     __syncthreads();
-#pragma unroll 2
+    const int low = s_low;
+    for (int i = threadIdx.x; i < count; i += kQuantThreads) s_entry[i] = low + i < n ? idx[low + i] : 0x7fffffff;
+    __syncthreads();
+    for (int j = threadIdx.x; j < count; j += kQuantThreads) {
+        const int t = (int)t_first + j;
+        int below = 0;                            // entries below token t
+        while (below < count && s_entry[below] < t) ++below;
+        s_row[j] = (below < count && s_entry[below] == t) ? low + below : -(t - low - below) - 1;
+    }
+    __syncthreads();
+
+#pragma unroll 1
     for (int it = 0; it < kQuantIters; ++it) {
-        const long long p = p0 + (long long)it * kPairsPerIter + (threadIdx.x >> 5) * kGroups + lane / kLanes;
-        const bool live = p < n_pairs;
-        const int t = live ? (int)(p / a.Hkv) : t_first, g = live ? (int)(p % a.Hkv) : 0;
-        const int where = s_row[t - t_first];
-        const bool in_T = where >= 0;
-        const int bits = in_T ? 4 : 2;
-        const int row = in_T ? where : -where - 1;         // its row in the "hi" / "lo" block
-        const bool fits = live && row < (in_T ? qb.cap_hi : qb.cap_lo);
-        float xk[8], xv[8];
-        if (live) {
-            const long long off = (long long)t * a.kv_stride + (long long)g * D + lg * 8;
-            unpack8s<kHalf>(*reinterpret_cast<const uint4 *>(k + off), xk);
-            unpack8s<kHalf>(*reinterpret_cast<const uint4 *>(v + off), xv);
-        } else {
+        if (p0 + it * kQuantPairs + (threadIdx.x >> 5) * 8 >= n_pairs) break;      // (the warp's first pair)
+        int row[2], bits[2];
+        long long rh[2];
+        bool fits[2];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) { xk[e] = 0.f; xv[e] = 0.f; }
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t p = pair_of(it, half);
+            const bool live = p < n_pairs;
+            const uint32_t j = live ? token_of(p) : 0, h = live ? p - p0 + g_first - j * (uint32_t)a.Hkv : 0;
+            const int where = s_row[j];
+            bits[half] = where >= 0 ? 4 : 2;
+            row[half] = where >= 0 ? where : -where - 1;
+            fits[half] = live && row[half] >= 0 && row[half] < (where >= 0 ? qb.cap_hi : qb.cap_lo);
+            rh[half] = (long long)row[half] * a.Hkv + h;
         }
-        unsigned short ks, kz, vs, vz;
-        const uint32_t ck = quantise8<kHalf, kLanes>(xk, bits, &ks, &kz);
-        const uint32_t cv = quantise8<kHalf, kLanes>(xv, bits, &vs, &vz);
-        if (fits) {
-            const long long rh = (long long)row * a.Hkv + g;
-            const int row_bytes = D * bits / 8;
-            store_codes((in_T ? qb.k_hi : qb.k_lo) + rh * row_bytes, lg, bits, ck);
-            store_codes((in_T ? qb.v_hi : qb.v_lo) + rh * row_bytes, lg, bits, cv);
-            if (lg == 0) {
-                unsigned short *pp = (in_T ? qb.p_hi : qb.p_lo) + rh * 4;
-                *reinterpret_cast<uint2 *>(pp) = make_uint2((uint32_t)ks | ((uint32_t)kz << 16),
-                                                            (uint32_t)vs | ((uint32_t)vz << 16));
+        // (max, -min) of each combination
+        uint32_t mm[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            uint32_t hi = w[u][0].x, lo = w[u][0].x;
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+                const uint32_t x[4] = {w[u][i].x, w[u][i].y, w[u][i].z, w[u][i].w};
+#pragma unroll
+                for (int e = (i == 0); e < 4; ++e) { hi = pk_max<kHalf>(hi, x[e]); lo = pk_min<kHalf>(lo, x[e]); }
             }
+            lo ^= 0x80008000u;
+            mm[u] = pk_max<kHalf>(__byte_perm(hi, lo, 0x5410), __byte_perm(hi, lo, 0x7632));
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) mm[u] = pk_max<kHalf>(mm[u], __shfl_xor_sync(0xffffffffu, mm[u], o));
+        // scale and reciprocal of combination lg & 3
+        const int mine = lg & 3;
+        const uint32_t m = mine == 0 ? mm[0] : mine == 1 ? mm[1] : mine == 2 ? mm[2] : mm[3];
+        const int my_bits = mine < 2 ? bits[0] : bits[1];
+        const float mx = storage_to_float<kHalf>((unsigned short)(m & 0xffffu));
+        const unsigned short zero_bits = (unsigned short)((m >> 16) ^ 0x8000u);
+        const float zero_mine = storage_to_float<kHalf>(zero_bits);
+        unsigned short scale_bits;
+        const float scale = storage_round<kHalf>(__fdiv_rn(__fsub_rn(mx, zero_mine), my_bits == 4 ? 15.f : 3.f), &scale_bits);
+        const float inv_mine = scale > 0.f ? __frcp_rn(scale) : 0.f;
+        // A scale that is no normal number of its type (its rounding error may take a code past the
+        // last level), a row with a NaN or an infinity: the quantiser of the append, step by step
+        const float smallest = kHalf ? 6.103515625e-5f : 1.17549435e-38f;
+        const bool odd = !(scale >= smallest && scale < 3e38f) && !(mx == zero_mine);
+        if (__any_sync(0xffffffffu, odd || mx != mx || fabsf(mx) > 3.3e38f || fabsf(zero_mine) > 3.3e38f)) {
+#pragma unroll 1
+            for (int u = 0; u < 4; ++u) {
+                const int bt = u < 2 ? bits[0] : bits[1];
+                float x[P][8];
+                for (int e = 0; e < P; ++e) unpack8s<kHalf>(u == 0 ? w[0][e] : u == 1 ? w[1][e] : u == 2 ? w[2][e] : w[3][e], x[e]);
+                uint32_t packed[P];
+                unsigned short sb, zb;
+                quantise<kHalf, 8, P>(x, bt, packed, &sb, &zb);
+                if (u < 2 ? fits[0] : fits[1]) {
+                    unsigned char *base = (u & 1) ? (bt == 4 ? qb.v_hi : qb.v_lo) : (bt == 4 ? qb.k_hi : qb.k_lo);
+                    const long long r = u < 2 ? rh[0] : rh[1];
+                    for (int e = 0; e < P; ++e) store_codes(base + r * (D * bt / 8), e * 8 + lg, bt, packed[e]);
+                    if (lg == 0) reinterpret_cast<uint32_t *>((bt == 4 ? qb.p_hi : qb.p_lo) + r * 4)[u & 1] = (uint32_t)sb | ((uint32_t)zb << 16);
+                }
+            }
+            if (it + 1 < kQuantIters) load(it + 1);
+            continue;
+        }
+        if (lg < 4 && (mine < 2 ? fits[0] : fits[1]))
+            reinterpret_cast<uint32_t *>((my_bits == 4 ? qb.p_hi : qb.p_lo) + (mine < 2 ? rh[0] : rh[1]) * 4)[mine & 1] =
+                (uint32_t)scale_bits | ((uint32_t)zero_bits << 16);
+        uint32_t code[4][P];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float inv = __shfl_sync(0xffffffffu, inv_mine, (lane & ~7) | u);
+            const float neg = storage_to_float<kHalf>((unsigned short)(mm[u] >> 16));      // -zero
+            const uint32_t mul = bits[u >> 1] == 4 ? 16u : 4u;
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+                float x[8];
+                unpack8s<kHalf>(w[u][i], x);
+                uint32_t acc = 0;
+#pragma unroll
+                for (int e = 7; e >= 0; --e)
+                    acc = acc * mul + __float_as_uint(__fadd_rn(__fmul_rn(__fadd_rn(x[e], neg), inv), 12582912.f));
+                // (the magic number's bits, 0x4B400000, of eight terms add up to this; 2-bit words keep 16 bits)
+                code[u][i] = acc - 0x3F400000u;
+            }
+        }
+        if (it + 1 < kQuantIters) load(it + 1);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int h = u >> 1;
+            if (!fits[h]) continue;
+            const bool hi4 = bits[h] == 4;
+            unsigned char *base = (u & 1) ? (hi4 ? qb.v_hi : qb.v_lo) : (hi4 ? qb.k_hi : qb.k_lo);
+#pragma unroll
+            for (int i = 0; i < P; ++i) store_codes(base + rh[h] * (hi4 ? D / 2 : D / 4), i * 8 + lg, hi4 ? 4 : 2, code[u][i]);
         }
     }
 }
@@ -107,7 +239,7 @@ zipvl_status run_quantize(const LayerArgs &a, const void *k, const void *v, cons
                           const int32_t *k_dev, int k_max, const QuantBlocks &qb, int32_t *lens_out,
                           int32_t *status_word, cudaStream_t st) {
     const long long pairs = (long long)a.L * a.Hkv;
-    const int per_cta = (kQuantThreads / 32) * (32 / (D / 8)) * kQuantIters;
+    const int per_cta = kQuantPairs * kQuantIters;
     const long long grid = (pairs + per_cta - 1) / per_cta;
     const cudaError_t e = launch_dependent(quantize_kv_kernel<kHalf, D>, dim3((unsigned)grid), dim3(kQuantThreads), 0, st,
                                            a, (const unsigned short *)k, (const unsigned short *)v, idx, k_dev, k_max,

@@ -27,14 +27,16 @@ __device__ __forceinline__ void unpack8s(const uint4 r, float (&x)[8]) {
     else unpack8(r, x);
 }
 
-// One (row, head) group of kLanes adjacent lanes, eight channels per lane: the quantiser's
-// parameters (rounded to the storage type) and this lane's eight codes packed at `bits` each.
-template <bool kHalf, int kLanes>
-__device__ __forceinline__ uint32_t quantise8(const float (&x)[8], int bits, unsigned short *scale_bits,
-                                              unsigned short *zero_bits) {
-    float mn = x[0], mx = x[0];
+// One (row, head) group of kLanes adjacent lanes, 8 P channels per lane: the quantiser's
+// parameters (rounded to the storage type) and this lane's codes packed at `bits` each, eight to a word.
+template <bool kHalf, int kLanes, int P>
+__device__ __forceinline__ void quantise(const float (&x)[P][8], int bits, uint32_t (&packed)[P],
+                                         unsigned short *scale_bits, unsigned short *zero_bits) {
+    float mn = x[0][0], mx = x[0][0];
 #pragma unroll
-    for (int e = 1; e < 8; ++e) { mn = fminf(mn, x[e]); mx = fmaxf(mx, x[e]); }
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { mn = fminf(mn, x[i][e]); mx = fmaxf(mx, x[i][e]); }
 #pragma unroll
     for (int o = kLanes / 2; o > 0; o >>= 1) {
         mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
@@ -43,16 +45,16 @@ __device__ __forceinline__ uint32_t quantise8(const float (&x)[8], int bits, uns
     const float levels = (float)((1 << bits) - 1);
     const float scale = storage_round<kHalf>(__fdiv_rn(__fsub_rn(mx, mn), levels), scale_bits);
     const float zero = storage_round<kHalf>(mn, zero_bits);
-    uint32_t packed = 0;
-    if (scale > 0.f) {
-        const float inv = __frcp_rn(scale);             // one correctly rounded reciprocal per row
+    const float inv = scale > 0.f ? __frcp_rn(scale) : 0.f;             // one correctly rounded reciprocal per row
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        packed[i] = 0;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const float c = fminf(fmaxf(rintf(__fmul_rn(__fsub_rn(x[e], zero), inv)), 0.f), levels);
-            packed |= (uint32_t)c << (bits * e);
+            const float c = fminf(fmaxf(rintf(__fmul_rn(__fsub_rn(x[i][e], zero), inv)), 0.f), levels);
+            packed[i] |= (scale > 0.f ? (uint32_t)c : 0u) << (bits * e);
         }
     }
-    return packed;
 }
 
 // Writes one lane's eight codes (32 bits at 4 bits each, 16 at 2) and, from the group's first

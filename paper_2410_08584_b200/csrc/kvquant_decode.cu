@@ -113,16 +113,17 @@ struct NewRow {
     __device__ __forceinline__ uint32_t quantise(int lane, uint32_t &par) const {
         constexpr int kLanes = D / 8;
         const int lg = lane % kLanes, which = lane / kLanes;
-        float x[8];
-        unpack8s<kHalf>(*reinterpret_cast<const uint4 *>(((which & 1) ? v : k) + lg * 8), x);
+        float x[1][8];
+        unpack8s<kHalf>(*reinterpret_cast<const uint4 *>(((which & 1) ? v : k) + lg * 8), x[0]);
         unsigned short scale, zero;
-        const uint32_t codes = quantise8<kHalf, kLanes>(x, 4, &scale, &zero);
+        uint32_t codes[1];
+        kvq::quantise<kHalf, kLanes, 1>(x, 4, codes, &scale, &zero);
         par = (uint32_t)scale | ((uint32_t)zero << 16);
         if (which < 2) {
-            store_codes((which & 1) ? v_hi : k_hi, lg, 4, codes);
+            store_codes((which & 1) ? v_hi : k_hi, lg, 4, codes[0]);
             if (lg == 0) reinterpret_cast<uint32_t *>(p_hi)[which] = par;
         }
-        return codes;
+        return codes[0];
     }
 };
 

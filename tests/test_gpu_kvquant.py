@@ -203,3 +203,36 @@ def test_quantised_decode_at_the_edges_of_its_steps(zipvl, n_hi, n_lo, Hq, Hkv, 
         assert err < (2e-3 if storage == "f16" else 8e-3), err
     assert st.item() == 0 and cache.lens.tolist() == [n_hi + 2, n_lo]
     _check_blocks(_blocks_from_gpu(cache, n_hi + 2, n_lo), ref)
+
+
+@pytest.mark.parametrize("L,H,d,dtype,keep", [(1, 1, 64, torch.bfloat16, 1.0), (129, 1, 128, torch.float16, 0.5),
+                                              (517, 3, 64, torch.float16, 0.0), (64, 40, 128, torch.bfloat16, 0.9),
+                                              (1031, 7, 128, torch.bfloat16, 0.03)])
+def test_quantiser_at_ragged_sizes_and_odd_values(zipvl, L, H, d, dtype, keep):
+    """Sizes that do not fill a CTA's pairs, token sets from empty to full, rows of equal values, of tiny values
+    (subnormal scales in fp16) and of values near the type's largest."""
+    z = zipvl
+    storage = "f16" if dtype == torch.float16 else "bf16"
+    g = torch.Generator().manual_seed(L + H)
+    k, v = torch.randn(L, H, d, generator=g), torch.randn(L, H, d, generator=g)
+    k[::5] = 0.25
+    v[1::7] *= 1e-6 if storage == "f16" else 1e-30
+    v[3::9] *= 1.5e4
+    k, v = k.to(dtype), v.to(dtype)
+    n = int(keep * L)
+    T = torch.sort(torch.randperm(L, generator=g)[:n]).values
+    idx = torch.full((L,), -1, dtype=torch.int32)
+    idx[:n] = T.to(torch.int32)
+    cache = z.QuantCache(L, H, d, dtype, DEV, cap_hi=n + 1, cap_lo=L - n + 1)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    lens = z.zipvl_quantize_kv(z.layer_desc(k, k), k.to(DEV), v.to(DEV), idx.to(DEV),
+                               torch.tensor([n], dtype=torch.int32, device=DEV), L, cache, status=st)
+    assert lens.tolist() == [n, L - n] and st.item() == 0
+    ref = oracle.quantize_kv(to_np(k), to_np(v), T.numpy(), storage)
+    got = _blocks_from_gpu(cache, n, L - n)
+    for name in ("hi", "lo"):
+        b = ref[name]
+        for t in "kv":
+            assert np.array_equal(got[name][t], oracle.pack_codes(b[f"{t}_codes"], b["bits"])), (name, t)
+            p = got[name]["p"][..., 0 if t == "k" else 2:][..., :2]
+            assert np.array_equal(p[..., 0], b[f"{t}_scale"]) and np.array_equal(p[..., 1], b[f"{t}_zero"])
