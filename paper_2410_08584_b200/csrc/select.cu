@@ -9,7 +9,8 @@
 //   top-p    the p-th largest ranking score u*; ties at u* go to the smaller
 //            position.
 // Rows of up to 4096 tokens run on one CTA that holds the row in registers (see
-// select_solo_kernel further down).  Longer rows: ceil(L / 1024) CTAs histogram 1024
+// select_solo_kernel further down), rows of up to 65536 on a cluster of eight (select_cluster_kernel).
+// Longer rows: ceil(L / 1024) CTAs histogram 1024
 // tokens each on the top 12 key bits (count and sum of the budget score, count of the
 // ranking score), add their
 // non-empty bins to a global histogram (64 KB of the workspace, cleared by a memset
@@ -19,6 +20,8 @@
 // position with one block-wide prefix sum.  The two searches are two passes of one
 // loop body.  Sums are 64-bit fixed point (2^-34 units, round to nearest), exact and
 // order independent, so the result repeats bit for bit.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace zipvl {
@@ -1065,6 +1068,501 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// Rows of 4097 to 65536 tokens: a cluster of eight CTAs, each with an eighth of the row in
+// registers and the histograms of its part in shared memory; the same searches as in
+// select_solo_kernel.  What bounds such a row is the chain of steps that the whole row has to take
+// together, so there are as few as possible: the parts' ranges, the level-1 histograms, and per search the
+// list of the tokens in the crossing bin -- four cluster barriers.  Everything between two
+// of them is done by every CTA for itself from the others' shared memory (first 256 sums of
+// 16 bins each, then the 16 bins of one of them), so nothing has to be handed back.  A
+// crossing bin with more tokens than the lists hold takes a further level (two barriers more).
+// The multi-CTA kernel above, which this replaces up to 65536 tokens, left everything behind the level-1
+// histogram to one CTA that walked the row five more times: 25 -> 16 us at 5003 tokens, 49 -> 20 us
+// at 18432, 125 -> 28 us at 32768.
+// ---------------------------------------------------------------------------------------
+constexpr int kClCtas = 8;
+constexpr int kClMax = 65536;
+constexpr int kClList = 64;                 // tokens of the crossing bin per CTA
+constexpr int kCoarse = kBins / 16;
+
+struct ClSmem : SoloSmem {
+    unsigned long long coarse_s[kCoarse];   // this CTA's sums over 16 bins
+    unsigned int coarse_c[kCoarse], coarse_r[kCoarse];
+    // what the other CTAs read
+    unsigned int range[4];                  // budget key {min, max}, ranking key {min, max}
+    unsigned long long sum, kept, all;
+    unsigned int n_list[2], above[2], list_key[2][kClList];     // per search: its own lists, so that no barrier
+    unsigned long long list_fx[2][kClList];                     // has to separate a reader from the next writer
+    unsigned int n_gt, n_eq, extra;
+    // the cluster's totals, for this CTA's search
+    unsigned long long tot_s[kCoarse];
+    unsigned int tot_c[kCoarse];
+    unsigned int all_key[kClCtas * kClList];
+    unsigned long long all_fx[kClCtas * kClList];
+};
+
+// The crossing bin over the whole cluster (level histograms `cnt` of all CTAs), as solo_find_bin.
+__device__ void cluster_find_bin(ClSmem &sm, bool by_sum, bool from_rank, unsigned long long target,
+                                 unsigned int carry_cnt, unsigned long long carry_sum, SoloCtl &c) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int t = threadIdx.x, lane = t & 31;
+    const unsigned int *coarse = from_rank ? sm.coarse_r : sm.coarse_c;
+    const unsigned int *fine = from_rank ? sm.cnt_r : sm.cnt;
+    if (t < kCoarse) {
+        unsigned int n = 0;
+        unsigned long long v = 0;
+#pragma unroll
+        for (int r = 0; r < kClCtas; ++r) n += *cl.map_shared_rank(coarse + t, r);
+        if (by_sum) {
+#pragma unroll
+            for (int r = 0; r < kClCtas; ++r) v += *cl.map_shared_rank(sm.coarse_s + t, r);
+        }
+        sm.tot_c[t] = n;
+        sm.tot_s[t] = v;
+    }
+    __syncthreads();
+    if (t < 32) {
+        // the group of 16 bins: eight groups per lane, from the top
+        unsigned int lc = 0;
+        unsigned long long ls = 0;
+#pragma unroll
+        for (int i = 0; i < kCoarse / 32; ++i) {
+            const int b = kCoarse - 1 - (lane * (kCoarse / 32) + i);
+            lc += sm.tot_c[b];
+            ls += sm.tot_s[b];
+        }
+        auto scan = [&](unsigned int &ic, unsigned long long &is) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int nc = __shfl_up_sync(0xffffffffu, ic, o);
+                const unsigned long long ns = __shfl_up_sync(0xffffffffu, is, o);
+                if (lane >= o) { ic += nc; is += ns; }
+            }
+        };
+        auto reached = [&](unsigned int rc, unsigned long long rs) {
+            return by_sum ? rs >= target : (unsigned long long)rc >= target;
+        };
+        unsigned int ic = lc;
+        unsigned long long is = ls;
+        scan(ic, is);
+        unsigned int run_c = carry_cnt + ic - lc;
+        unsigned long long run_s = carry_sum + is - ls;
+        unsigned int who = __ballot_sync(0xffffffffu, lc > 0 && reached(run_c + lc, run_s + ls));
+        if (who == 0) {
+            if (lane == 0) c.hit = 0xffffffffu;          // (no bin qualifies)
+        } else {
+            const int src = __ffs(who) - 1;
+            int group = 0;
+            if (lane == src) {
+                for (int i = 0; i < kCoarse / 32; ++i) {
+                    group = kCoarse - 1 - (lane * (kCoarse / 32) + i);
+                    const unsigned int n = sm.tot_c[group];
+                    if (n > 0 && reached(run_c + n, run_s + sm.tot_s[group])) break;
+                    run_c += n;
+                    run_s += sm.tot_s[group];
+                }
+            }
+            group = __shfl_sync(0xffffffffu, group, src);
+            run_c = __shfl_sync(0xffffffffu, run_c, src);
+            run_s = __shfl_sync(0xffffffffu, run_s, src);
+            // its 16 bins, from the top: lanes i and i + 16 add up four CTAs each
+            const int b = group * 16 + 15 - (lane & 15);
+            unsigned int n = 0;
+            unsigned long long v = 0;
+#pragma unroll
+            for (int r = 0; r < kClCtas / 2; ++r) {
+                const int from = (lane >> 4) * (kClCtas / 2) + r;
+                n += *cl.map_shared_rank(fine + b, from);
+                if (by_sum)
+                    v += (unsigned long long)*cl.map_shared_rank(&sm.sum16[0][b], from) +
+                         ((unsigned long long)*cl.map_shared_rank(&sm.sum16[1][b], from) << 16) +
+                         ((unsigned long long)*cl.map_shared_rank(&sm.sum16[2][b], from) << 32);
+            }
+            n += __shfl_xor_sync(0xffffffffu, n, 16);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            ic = lane < 16 ? n : 0;
+            is = lane < 16 ? v : 0;
+            scan(ic, is);
+            run_c += ic - n;
+            run_s += is - v;
+            who = __ballot_sync(0xffffffffu, lane < 16 && n > 0 && reached(run_c + n, run_s + v));
+            if (who && lane == __ffs(who) - 1) {
+                c.hit = 0;
+                c.hit_bin = (unsigned int)b;
+                c.cnt_gt = run_c;
+                c.sum_gt = run_s;
+                c.bin_cnt = n;
+                c.bin_sum = v;
+            }
+        }
+    }
+    __syncthreads();
+}
+
+template <bool kKeepLast, int kPer>
+__global__ void __launch_bounds__(kSoloThreads) __cluster_dims__(kClCtas, 1, 1)
+select_cluster_kernel(int L, const float *__restrict__ acc, const float *__restrict__ norm, float tau,
+                      uint32_t mode, int fixed_k, int32_t *__restrict__ k_out, int32_t *__restrict__ idx,
+                      float *__restrict__ kept_mass, int32_t *status_word) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char sel_dyn[];
+    ClSmem &sm = *reinterpret_cast<ClSmem *>(sel_dyn);
+    __shared__ SoloCtl c;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = blockIdx.x;
+    auto clear = [&](void *p, int bytes) {
+        uint4 *z = reinterpret_cast<uint4 *>(p);
+        for (int e = threadIdx.x; e < bytes / 16; e += kSoloThreads) z[e] = make_uint4(0, 0, 0, 0);
+    };
+    clear(&sm, sizeof(SoloSmem));      // while the previous kernel may still be running
+    if (threadIdx.x < 2) sm.n_list[threadIdx.x] = 0;
+    grid_launch_dependents();
+    grid_dependency_wait(acc, norm);   // the scores are the previous kernel's output
+    const size_t z = blockIdx.y;       // sequence of a batch
+    acc += z * L;
+    norm += z * L;
+    idx += z * L;
+    k_out += z;
+    if (kept_mass) kept_mass += z;
+    const bool bud_is_norm = (mode & ZIPVL_BUDGET_BY_NORM) != 0, rank_is_acc = (mode & ZIPVL_TOPK_BY_ACC) != 0;
+    // ---- this CTA's part of the row, kPer consecutive positions per thread ----
+    const int chunk = ((L + kClCtas - 1) / kClCtas + 3) & ~3;
+    const int j0 = rank * chunk + (int)threadIdx.x * kPer, j_end = min(L, (rank + 1) * chunk);
+    float av[kPer], nv[kPer];
+    const bool vec = (((uintptr_t)acc | (uintptr_t)norm) & 15u) == 0;
+#pragma unroll
+    for (int v4 = 0; v4 < kPer / 4; ++v4) {
+        const int j = j0 + 4 * v4;
+        if (vec && j + 4 <= j_end) {
+            const float4 a4 = *reinterpret_cast<const float4 *>(acc + j);
+            const float4 n4 = *reinterpret_cast<const float4 *>(norm + j);
+            av[4 * v4] = a4.x; av[4 * v4 + 1] = a4.y; av[4 * v4 + 2] = a4.z; av[4 * v4 + 3] = a4.w;
+            nv[4 * v4] = n4.x; nv[4 * v4 + 1] = n4.y; nv[4 * v4 + 2] = n4.z; nv[4 * v4 + 3] = n4.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                av[4 * v4 + e] = (j + e < j_end) ? acc[j + e] : 0.f;
+                nv[4 * v4 + e] = (j + e < j_end) ? norm[j + e] : 0.f;
+            }
+        }
+    }
+    unsigned int kb[kPer], kr[kPer];
+    unsigned int mn[2] = {0xffffffffu, 0xffffffffu}, mx[2] = {0u, 0u};
+    unsigned long long my_sum = 0;
+    bool bad_value = false;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        const float vb = bud_is_norm ? nv[e] : av[e], vr = rank_is_acc ? av[e] : nv[e];
+        kb[e] = float_key(vb);
+        kr[e] = float_key(vr);
+        if (j0 + e < j_end) {
+            mn[0] = min(mn[0], kb[e]); mx[0] = max(mx[0], kb[e]);
+            mn[1] = min(mn[1], kr[e]); mx[1] = max(mx[1], kr[e]);
+            my_sum += to_fx(vb);
+            bad_value |= !(vb >= 0.f) || !(vr >= 0.f);
+        }
+    }
+    if (bad_value) report(status_word, ZIPVL_DEV_BAD_VALUE);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        mn[x] = __reduce_min_sync(0xffffffffu, mn[x]);
+        mx[x] = __reduce_max_sync(0xffffffffu, mx[x]);
+        if (lane == 0) { c.wmin[x][warp] = mn[x]; c.wmax[x][warp] = mx[x]; }
+    }
+    {
+        unsigned int uc;
+        unsigned long long us, S;
+        solo_scan(0u, my_sum, c, &uc, &us, nullptr, &S);
+        if (threadIdx.x == 0) {
+            sm.sum = S;
+            for (int x = 0; x < 2; ++x) {
+                unsigned int lo = 0xffffffffu, hi = 0u;
+                for (int i = 0; i < kSoloWarps; ++i) { lo = min(lo, c.wmin[x][i]); hi = max(hi, c.wmax[x][i]); }
+                sm.range[2 * x] = lo;
+                sm.range[2 * x + 1] = hi;
+            }
+        }
+    }
+    cl.sync();                         // (1) ranges and sums are in; every CTA's histograms are clear
+    unsigned long long S_all = 0;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) { mn[x] = 0xffffffffu; mx[x] = 0u; }
+#pragma unroll
+    for (int r = 0; r < kClCtas; ++r) {
+        const unsigned int *o = cl.map_shared_rank(sm.range, r);
+        mn[0] = min(mn[0], o[0]); mx[0] = max(mx[0], o[1]);
+        mn[1] = min(mn[1], o[2]); mx[1] = max(mx[1], o[3]);
+        S_all += *cl.map_shared_rank(&sm.sum, r);
+    }
+    auto first_shift = [](unsigned int lo, unsigned int hi) {
+        const int bits = 32 - __clz(hi - lo);
+        return bits > 12 ? bits - 12 : 0;
+    };
+    const bool need_budget = !(fixed_k > 0) && (tau < 1.0f);
+    const int shift1[2] = {first_shift(mn[0], mx[0]), first_shift(mn[1], mx[1])};
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        if (j0 + e < j_end) {
+            if (need_budget) solo_add(sm, (kb[e] - mn[0]) >> shift1[0], to_fx(bud_is_norm ? nv[e] : av[e]));
+            atomicAdd(&sm.cnt_r[(kr[e] - mn[1]) >> shift1[1]], 1u);
+        }
+    }
+    // sums of 16 bins: the budget level by the first half of the threads, the ranking level by the second
+    auto coarsen = [&](bool budget_or_level, bool sums, bool ranking) {
+        __syncthreads();
+        const int t = threadIdx.x & (kCoarse - 1);
+        const bool second = threadIdx.x >= kCoarse;
+        if (second ? ranking : budget_or_level) {
+            const uint4 *src = reinterpret_cast<const uint4 *>((second ? sm.cnt_r : sm.cnt) + 16 * t);
+            unsigned int n = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { const uint4 q = src[i]; n += q.x + q.y + q.z + q.w; }
+            (second ? sm.coarse_r : sm.coarse_c)[t] = n;
+            if (!second) {
+                unsigned long long v = 0;
+                if (sums && n)
+                    for (int i = 0; i < 16; ++i) v += solo_sum(sm, 16 * t + i);
+                sm.coarse_s[t] = v;
+            }
+        }
+    };
+    static_assert(kSoloThreads == 2 * kCoarse, "one thread per group of bins and level");
+    coarsen(need_budget, true, true);
+    cl.sync();                         // (2) the level-1 histograms
+    unsigned int p = (fixed_k > 0) ? (unsigned int)min(fixed_k, L) : (unsigned int)L;
+    unsigned int thr_key = 0, need_eq = L;
+    bool counted = false;              // n_gt / n_eq of every CTA follow from the lists of the ranking search
+#pragma unroll 1
+    for (int pass = need_budget ? 0 : 1; pass < 2; ++pass) {
+        const bool by_sum = (pass == 0);
+        if (!by_sum && p >= (unsigned int)L) break;
+        const unsigned int *keys = by_sum ? kb : kr;
+        const unsigned long long target = by_sum ? (unsigned long long)ceil((double)tau * (double)S_all) : (unsigned long long)p;
+        unsigned int base = mn[pass], carry_c = 0;
+        unsigned long long carry_s = 0;
+        int shift = shift1[pass], width_log2 = 32;
+        bool found = true;
+#pragma unroll 1
+        for (int level = 0;; ++level) {
+            if (level > 0) {
+                // 4096 bins over the crossing bin of the level before
+                cl.sync();             // nobody reads the old histogram any more
+                clear(sm.cnt, sizeof(sm.cnt));
+                if (by_sum) clear(sm.sum16, sizeof(sm.sum16));
+                if (threadIdx.x == 0) sm.n_list[pass] = 0;
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < kPer; ++e) {
+                    unsigned int d;
+                    if (j0 + e < j_end && solo_bin(keys[e], base, width_log2, shift, &d)) {
+                        if (by_sum) solo_add(sm, d, to_fx(bud_is_norm ? nv[e] : av[e]));
+                        else atomicAdd(&sm.cnt[d], 1u);
+                    }
+                }
+                coarsen(true, by_sum, false);
+                cl.sync();
+            }
+            cluster_find_bin(sm, by_sum, !by_sum && level == 0, target, carry_c, carry_s, c);
+            if (c.hit == 0xffffffffu) { found = false; break; }     // (rounding let no prefix qualify)
+            if (shift == 0) { thr_key = base + c.hit_bin; break; }  // the bin is one key value
+            // the tokens of the crossing bin, and how many lie above it
+            const unsigned int bin_lo = base + (c.hit_bin << shift), bin_hi = bin_lo + ((1u << shift) - 1u);
+            unsigned int above = 0;
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) {
+                if (j0 + e < j_end) {
+                    above += keys[e] > bin_hi;
+                    if (keys[e] >= bin_lo && keys[e] <= bin_hi && c.bin_cnt <= kClCtas * kClList) {
+                        const unsigned int slot = atomicAdd(&sm.n_list[pass], 1u);
+                        if (slot < kClList) {
+                            sm.list_key[pass][slot] = keys[e];
+                            sm.list_fx[pass][slot] = by_sum ? to_fx(bud_is_norm ? nv[e] : av[e]) : 0ull;
+                        }
+                    }
+                }
+            }
+            above = __reduce_add_sync(0xffffffffu, above);
+            if (lane == 0) c.wcnt[warp] = above;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                unsigned int n = 0;
+                for (int i = 0; i < kSoloWarps; ++i) n += c.wcnt[i];
+                sm.above[pass] = n;
+            }
+            cl.sync();                 // (3), (4) the lists
+            unsigned int n_of = lane < kClCtas ? *cl.map_shared_rank(&sm.n_list[pass], lane) : 0u;
+            const bool listed = c.bin_cnt <= kClCtas * kClList && !__any_sync(0xffffffffu, n_of > kClList);
+            if (listed) {
+                unsigned int before = n_of;                          // entries of the CTAs in front
+#pragma unroll
+                for (int o = 1; o < kClCtas; o <<= 1) {
+                    const unsigned int x = __shfl_up_sync(0xffffffffu, before, o);
+                    if (lane >= o) before += x;
+                }
+                const unsigned int n_all = __shfl_sync(0xffffffffu, before, kClCtas - 1);
+                before -= n_of;
+                if (warp < kClCtas) {
+                    const unsigned int off = __shfl_sync(0xffffffffu, before, warp), n = __shfl_sync(0xffffffffu, n_of, warp);
+                    for (unsigned int i = lane; i < n; i += 32) {
+                        sm.all_key[off + i] = *cl.map_shared_rank(&sm.list_key[pass][i], warp);
+                        sm.all_fx[off + i] = *cl.map_shared_rank(&sm.list_fx[pass][i], warp);
+                    }
+                }
+                const unsigned int above_c = c.cnt_gt;
+                const unsigned long long above_s = c.sum_gt;
+                __syncthreads();
+                if (threadIdx.x < n_all) {
+                    const unsigned int my_key = sm.all_key[threadIdx.x];
+                    unsigned int gt_c = 0, eq_c = 0;
+                    unsigned long long gt_s = 0;
+                    for (unsigned int o = 0; o < n_all; ++o) {
+                        const unsigned int ko = sm.all_key[o];
+                        if (ko > my_key) { ++gt_c; gt_s += sm.all_fx[o]; }
+                        eq_c += (ko == my_key);
+                    }
+                    const unsigned long long eq_s = sm.all_fx[threadIdx.x] * eq_c;
+                    bool hit;
+                    if (by_sum) hit = (above_s + gt_s + eq_s >= target) && (gt_c == 0 || above_s + gt_s < target);
+                    else hit = ((unsigned long long)above_c + gt_c + eq_c >= target) &&
+                               (gt_c == 0 || (unsigned long long)above_c + gt_c < target);
+                    if (hit) {                                       // (copies of one key write the same values)
+                        c.cnt_gt = above_c + gt_c;
+                        c.sum_gt = above_s + gt_s;
+                        c.bin_cnt = eq_c;
+                        c.bin_sum = eq_s;
+                        c.one_key = my_key;
+                    }
+                }
+                __syncthreads();
+                thr_key = c.one_key;
+                counted = !by_sum;
+                break;
+            }
+            base = bin_lo;
+            carry_c = c.cnt_gt;
+            carry_s = c.sum_gt;
+            width_log2 = shift;
+            shift = shift > 12 ? shift - 12 : 0;
+        }
+        if (by_sum) {
+            if (found) {
+                // copies of the threshold value enter one at a time
+                const unsigned long long v = c.bin_cnt ? c.bin_sum / c.bin_cnt : 0ull;
+                unsigned long long need = 1;
+                if (target > c.sum_gt && v > 0) need = (target - c.sum_gt + v - 1) / v;
+                if (need < 1) need = 1;
+                if (need > c.bin_cnt) need = c.bin_cnt;
+                p = c.cnt_gt + (unsigned int)need;
+            }
+            thr_key = 0;
+            __syncthreads();           // (c is rewritten by the next search)
+        } else {
+            need_eq = p - c.cnt_gt;
+        }
+    }
+
+    // ---- emit T ascending from the registers ----
+    const bool all_sel = (p >= (unsigned int)L);
+    unsigned int n_gt = 0, n_eq = 0;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        if (j0 + e < j_end) {
+            n_gt += kr[e] > thr_key;
+            n_eq += kr[e] == thr_key;
+        }
+    }
+    unsigned int eq_before, eq_here;
+    unsigned long long gt_before, gt_here;
+    solo_scan(n_eq, (unsigned long long)n_gt, c, &eq_before, &gt_before, &eq_here, &gt_here);
+    if (!all_sel) {
+        // what the CTAs in front hold
+        if (!counted) {
+            if (threadIdx.x == 0) { sm.n_gt = (unsigned int)gt_here; sm.n_eq = eq_here; }
+            cl.sync();
+        }
+        unsigned int g = 0, q = 0;
+        if (lane < rank) {
+            if (counted) {
+                g = *cl.map_shared_rank(&sm.above[1], lane);
+                const unsigned int n = *cl.map_shared_rank(&sm.n_list[1], lane);
+                for (unsigned int i = 0; i < n; ++i) {
+                    const unsigned int ko = *cl.map_shared_rank(&sm.list_key[1][i], lane);
+                    g += ko > thr_key;
+                    q += ko == thr_key;
+                }
+            } else {
+                g = *cl.map_shared_rank(&sm.n_gt, lane);
+                q = *cl.map_shared_rank(&sm.n_eq, lane);
+            }
+        }
+        gt_before += __reduce_add_sync(0xffffffffu, g);
+        eq_before += __reduce_add_sync(0xffffffffu, q);
+    }
+    const unsigned int eq_take = all_sel ? n_eq : min(n_eq, need_eq > eq_before ? need_eq - eq_before : 0u);
+    unsigned int out = all_sel ? (unsigned int)min(j0, j_end) : (unsigned int)gt_before + min(eq_before, need_eq);
+    unsigned int tot_sel = all_sel ? (unsigned int)L : p;
+    const unsigned int keep_last = mode >> 8;
+    const int f0 = (kKeepLast && keep_last > 0 && !all_sel) ? max(0, L - (int)min(keep_last, (unsigned int)L)) : L;
+    if (kKeepLast && f0 < L) {
+        // the final positions the threshold leaves out, in front of this thread and in all
+        unsigned int extra = 0, left = eq_take;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            if (j0 + e < j_end) {
+                bool keep = kr[e] > thr_key;
+                if (!keep && kr[e] == thr_key && left > 0) { keep = true; --left; }
+                extra += (!keep && j0 + e >= f0);
+            }
+        }
+        unsigned int extra_before, extra_here;
+        unsigned long long unused;
+        solo_scan(extra, 0ull, c, &extra_before, &unused, &extra_here);
+        if (threadIdx.x == 0) sm.extra = extra_here;
+        cl.sync();
+        const unsigned int x = lane < kClCtas ? *cl.map_shared_rank(&sm.extra, lane) : 0u;
+        out += extra_before + __reduce_add_sync(0xffffffffu, lane < rank ? x : 0u);
+        tot_sel += __reduce_add_sync(0xffffffffu, x);
+    }
+    unsigned int eq_left = eq_take;
+    unsigned long long mass = 0, all = 0;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        const int j = j0 + e;
+        if (j < j_end) {
+            bool keep = true;
+            if (!all_sel) {
+                keep = kr[e] > thr_key;
+                if (!keep && kr[e] == thr_key && eq_left > 0) { keep = true; --eq_left; }
+                if (kKeepLast) keep = keep || (j >= f0);
+            }
+            if (kept_mass) {
+                const unsigned long long fx = to_fx(av[e]);
+                all += fx;
+                if (keep) mass += fx;
+            }
+            if (keep) idx[out++] = j;
+        }
+    }
+    for (int j = (int)tot_sel + rank * kSoloThreads + (int)threadIdx.x; j < L; j += kClCtas * kSoloThreads) idx[j] = -1;
+    if (rank == 0 && threadIdx.x == 0) *k_out = (int32_t)tot_sel;
+    if (kept_mass) {
+        unsigned int uc;
+        unsigned long long us, kept, S_acc;
+        solo_scan(0u, mass, c, &uc, &us, nullptr, &kept);
+        solo_scan(0u, all, c, &uc, &us, nullptr, &S_acc);
+        if (threadIdx.x == 0) { sm.kept = kept; sm.all = S_acc; }
+        cl.sync();
+        if (rank == 0 && threadIdx.x == 0) {
+            kept = 0; S_acc = 0;
+            for (int r = 0; r < kClCtas; ++r) { kept += *cl.map_shared_rank(&sm.kept, r); S_acc += *cl.map_shared_rank(&sm.all, r); }
+            *kept_mass = S_acc ? (float)((double)kept / (double)S_acc) : 0.f;
+        }
+    }
+    cl.sync();                         // nobody leaves while its shared memory is read
+}
+
 }  // namespace
 
 size_t select_ws_bytes() { return (sizeof(GlobalHist) + 255) & ~(size_t)255; }
@@ -1072,8 +1570,8 @@ size_t select_ws_bytes() { return (sizeof(GlobalHist) + 255) & ~(size_t)255; }
 zipvl_status launch_select(int L, const float *acc, const float *norm, float tau, uint32_t mode,
                            int fixed_k, int32_t *k_out, int32_t *idx, float *kept_mass, void *ws,
                            int32_t *status_word, cudaStream_t st, int n_seq) {
-    if (L > kSoloMax && n_seq > 1) {
-        // long rows: the multi-CTA kernel takes one sequence at a time (its workspace too)
+    if (L > kClMax && n_seq > 1) {
+        // the longest rows: the multi-CTA kernel takes one sequence at a time (its workspace too)
         for (int z = 0; z < n_seq; ++z) {
             const zipvl_status sz = launch_select(L, acc + (size_t)z * L, norm + (size_t)z * L, tau, mode, fixed_k,
                                                   k_out + z, idx + (size_t)z * L, kept_mass ? kept_mass + z : nullptr,
@@ -1090,6 +1588,19 @@ zipvl_status launch_select(int L, const float *acc, const float *norm, float tau
             es = launch_dependent(solo, dim3(n_seq), dim3(kSoloThreads), sizeof(SoloSmem), st, L, acc, norm, tau,
                                   mode, fixed_k, k_out, idx, kept_mass, status_word);
         if (es != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "select: launch: %s", cudaGetErrorString(es));
+        count_launches(1);
+        return check_launch("zipvl_select");
+    }
+    if (L <= kClMax) {
+        // a cluster per sequence; 4, 8 or 16 positions per thread
+        auto *cluster = L <= kClCtas * kSoloThreads * 4   ? ((mode >> 8) ? select_cluster_kernel<true, 4> : select_cluster_kernel<false, 4>)
+                        : L <= kClCtas * kSoloThreads * 8 ? ((mode >> 8) ? select_cluster_kernel<true, 8> : select_cluster_kernel<false, 8>)
+                                                          : ((mode >> 8) ? select_cluster_kernel<true, 16> : select_cluster_kernel<false, 16>);
+        cudaError_t ec = cudaFuncSetAttribute(cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClSmem));
+        if (ec == cudaSuccess)
+            ec = launch_dependent(cluster, dim3(kClCtas, n_seq), dim3(kSoloThreads), sizeof(ClSmem), st, L, acc, norm, tau,
+                                  mode, fixed_k, k_out, idx, kept_mass, status_word);
+        if (ec != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "select: launch: %s", cudaGetErrorString(ec));
         count_launches(1);
         return check_launch("zipvl_select");
     }
