@@ -4,7 +4,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
@@ -35,7 +34,7 @@ void count_launches(int n) { __atomic_fetch_add(&g_launches, (unsigned long long
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-static zipvl_status check_layer(const char *who, const zipvl_layer *l, LayerArgs *a) {
+zipvl_status check_layer(const char *who, const zipvl_layer *l, LayerArgs *a) {
     if (!l) return fail(ZIPVL_ERR_INVALID_ARG, "%s: layer is NULL", who);
     if (l->L < 1) return fail(ZIPVL_ERR_INVALID_ARG, "%s: L = %d < 1", who, l->L);
     if (l->n_q_heads < 1 || l->n_kv_heads < 1 || l->n_q_heads % l->n_kv_heads)
@@ -57,11 +56,10 @@ static zipvl_status check_layer(const char *who, const zipvl_layer *l, LayerArgs
     const float scale = l->softmax_scale > 0.f ? l->softmax_scale : 1.0f / sqrtf((float)l->head_dim);
     a->scale_log2 = scale * kLog2e;
     a->half = (l->dtype == ZIPVL_F16);
-    a->n_seq = 1; a->q_seq = 0; a->kv_seq = 0;
+    a->n_seq = 1; a->q_seq = 0; a->kv_seq = 0; a->h0 = 0; a->hn = l->n_q_heads;
     return ZIPVL_OK;
 }
 
-static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace zipvl
 
@@ -383,169 +381,6 @@ zipvl_status zipvl_sparse_prefill_batch(const zipvl_layer *layer, const zipvl_ba
         if (s != ZIPVL_OK) return s;
     }
     return ZIPVL_OK;
-}
-
-#define ZIPVL_CUDA(call)                                                                   \
-    do {                                                                                   \
-        cudaError_t e_ = (call);                                                           \
-        if (e_ != cudaSuccess) {                                                           \
-            st_ = fail(ZIPVL_ERR_CUDA, "prefill_layer_host: %s: %s", #call, cudaGetErrorString(e_)); \
-            goto done;                                                                     \
-        }                                                                                  \
-    } while (0)
-
-namespace {
-// Device scratch of zipvl_prefill_layer_host comes from a memory pool of the library's own
-// (one per device, created on first use) whose release threshold is unlimited: the
-// few hundred MB a call needs are then handed back to the pool, not to the driver, when
-// the call ends, and the next call gets them again at once.  With the device's default
-// pool every call paid for mapping and unmapping that memory (16 ms against 2.7 ms per
-// call on a 2944-token layer).  zipvl_release_host_scratch() gives the memory back.
-constexpr int kMaxDevices = 64;
-cudaMemPool_t g_host_pool[kMaxDevices] = {};
-std::mutex g_host_pool_mutex;   // two first calls on one device must not both create a pool
-
-cudaError_t host_pool(cudaMemPool_t *pool) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_host_pool_mutex);
-    if (!g_host_pool[dev]) {
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t p = nullptr;
-        e = cudaMemPoolCreate(&p, &props);
-        if (e != cudaSuccess) return e;
-        unsigned long long keep = ~0ull;
-        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (e != cudaSuccess) { cudaMemPoolDestroy(p); return e; }
-        g_host_pool[dev] = p;
-    }
-    *pool = g_host_pool[dev];
-    return cudaSuccess;
-}
-}  // namespace
-
-zipvl_status zipvl_release_host_scratch(void) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
-        return fail(ZIPVL_ERR_CUDA, "zipvl_release_host_scratch: no current device");
-    std::lock_guard<std::mutex> lock(g_host_pool_mutex);
-    if (g_host_pool[dev]) {
-        const cudaError_t e = cudaMemPoolTrimTo(g_host_pool[dev], 0);
-        if (e != cudaSuccess)
-            return fail(ZIPVL_ERR_CUDA, "zipvl_release_host_scratch: %s", cudaGetErrorString(e));
-    }
-    return ZIPVL_OK;
-}
-
-zipvl_status zipvl_prefill_layer_host(const zipvl_layer *layer, const void *q, const void *k,
-                                      const void *v, const int32_t *probe_pos, int32_t n_probe,
-                                      float tau, int32_t *k_out, int32_t *idx_out, void *out,
-                                      void *k_cache_out, void *v_cache_out) {
-    return zipvl_layer_step_host(layer, q, k, v, probe_pos, n_probe, tau, k_out, idx_out, out,
-                                 k_cache_out, v_cache_out, nullptr, nullptr, nullptr, nullptr);
-}
-
-zipvl_status zipvl_layer_step_host(const zipvl_layer *layer, const void *q, const void *k,
-                                   const void *v, const int32_t *probe_pos, int32_t n_probe,
-                                   float tau, int32_t *k_out, int32_t *idx_out, void *out,
-                                   void *k_cache_out, void *v_cache_out, const void *q_new,
-                                   const void *k_new, const void *v_new, void *decode_out) {
-    LayerArgs a{};
-    zipvl_status st_ = check_layer("zipvl_layer_step_host", layer, &a);
-    if (st_ != ZIPVL_OK) return st_;
-    if (!q || !k || !v || !probe_pos || n_probe < 1)
-        return fail(ZIPVL_ERR_INVALID_ARG, "zipvl_layer_step_host: NULL input or n_probe < 1");
-    if (layer->q_stride_tok || layer->kv_stride_tok)
-        return fail(ZIPVL_ERR_UNSUPPORTED, "zipvl_layer_step_host: contiguous tensors only");
-    const bool with_decode = (q_new != nullptr);
-    if (with_decode && (!k_new || !v_new || !decode_out))
-        return fail(ZIPVL_ERR_INVALID_ARG, "zipvl_layer_step_host: the decode step needs q_new, k_new, v_new and decode_out");
-    if (with_decode && a.G > 8)
-        return fail(ZIPVL_ERR_UNSUPPORTED, "zipvl_layer_step_host: more than 8 query heads per kv head");
-    const size_t eb = elem_bytes(layer->dtype);
-    const size_t qb = (size_t)a.L * a.Hq * a.D * eb, kb = (size_t)a.L * a.Hkv * a.D * eb;
-    const size_t ws_score = zipvl_workspace_bytes(ZIPVL_OP_SCORE, layer, n_probe, 1);
-    const size_t ws_pf = zipvl_workspace_bytes(ZIPVL_OP_SPARSE_PREFILL, layer, 0, 1);
-    size_t ws_b = ws_score > ws_pf ? ws_score : ws_pf;
-    if (ws_b < select_ws_bytes()) ws_b = select_ws_bytes();
-    // the decode step runs on the cache this call has just compacted: capacity L + 1 rows
-    const size_t ws_dec = with_decode ? align256(decode_ws_bytes(1, a.Hq, a.D, a.L + 1, a.Hkv, layer->dtype)) : 0;
-    if (ws_b < ws_dec) ws_b = ws_dec;
-    const size_t qn_b = (size_t)a.Hq * a.D * eb, kn_b = (size_t)a.Hkv * a.D * eb;
-    // one stream-ordered allocation carved into pieces
-    size_t off = 0;
-    auto carve = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
-    const size_t o_q = carve(qb), o_k = carve(kb), o_v = carve(kb), o_out = carve(qb),
-                 o_kc = carve(kb + kn_b), o_vc = carve(kb + kn_b), o_probe = carve((size_t)n_probe * 4),
-                 o_qn = carve(qn_b), o_kn = carve(kn_b), o_vn = carve(kn_b), o_dec = carve(qn_b),
-                 o_acc = carve((size_t)a.L * 4), o_norm = carve((size_t)a.L * 4),
-                 o_idx = carve((size_t)a.L * 4), o_misc = carve(256), o_ws = carve(ws_b);
-    char *base = nullptr;
-    cudaStream_t s = nullptr;
-    cudaMemPool_t pool = nullptr;
-    int32_t misc[4] = {0, 0, 0, 0};   // k, cache length, device status word, (cache capacity)
-    ZIPVL_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-    ZIPVL_CUDA(host_pool(&pool));
-    ZIPVL_CUDA(cudaMallocFromPoolAsync((void **)&base, off, pool, s));
-    {
-        int32_t *d_misc = (int32_t *)(base + o_misc);  // [0] k, [1] len, [2] status
-        ZIPVL_CUDA(cudaMemsetAsync(d_misc, 0, 256, s));
-        ZIPVL_CUDA(cudaMemcpyAsync(base + o_q, q, qb, cudaMemcpyHostToDevice, s));
-        ZIPVL_CUDA(cudaMemcpyAsync(base + o_k, k, kb, cudaMemcpyHostToDevice, s));
-        ZIPVL_CUDA(cudaMemcpyAsync(base + o_v, v, kb, cudaMemcpyHostToDevice, s));
-        ZIPVL_CUDA(cudaMemcpyAsync(base + o_probe, probe_pos, (size_t)n_probe * 4, cudaMemcpyHostToDevice, s));
-        if (with_decode) {
-            ZIPVL_CUDA(cudaMemcpyAsync(base + o_qn, q_new, qn_b, cudaMemcpyHostToDevice, s));
-            ZIPVL_CUDA(cudaMemcpyAsync(base + o_kn, k_new, kn_b, cudaMemcpyHostToDevice, s));
-            ZIPVL_CUDA(cudaMemcpyAsync(base + o_vn, v_new, kn_b, cudaMemcpyHostToDevice, s));
-        }
-        st_ = zipvl_score(layer, base + o_q, base + o_k, (int32_t *)(base + o_probe), n_probe,
-                          (float *)(base + o_acc), (float *)(base + o_norm), nullptr, base + o_ws,
-                          ws_b, d_misc + 2, s);
-        if (st_ != ZIPVL_OK) goto done;
-        st_ = zipvl_select(a.L, (float *)(base + o_acc), (float *)(base + o_norm), tau, 0, 0, d_misc,
-                           (int32_t *)(base + o_idx), nullptr, base + o_ws, ws_b, d_misc + 2, s);
-        if (st_ != ZIPVL_OK) goto done;
-        st_ = zipvl_sparse_prefill_compact(layer, base + o_q, base + o_k, base + o_v,
-                                           (int32_t *)(base + o_idx), d_misc, a.L, base + o_out,
-                                           ZIPVL_OUT_PADDED, base + o_kc, base + o_vc, a.L, d_misc + 1,
-                                           base + o_ws, ws_b, d_misc + 2, s);
-        if (st_ != ZIPVL_OK) goto done;
-        if (with_decode) {
-            // Algorithm 2 on the cache just built: d_misc[1] holds its length, d_misc[3] its
-            // capacity, d_misc + 4 (8-byte aligned) the one request's offset 0
-            const int32_t cap = a.L + 1;
-            ZIPVL_CUDA(cudaMemcpyAsync(d_misc + 3, &cap, 4, cudaMemcpyHostToDevice, s));
-            zipvl_decode_desc dd = {1, a.Hq, a.Hkv, a.D, layer->dtype, layer->softmax_scale};
-            st_ = zipvl_decode(&dd, base + o_qn, base + o_kn, base + o_vn, base + o_kc, base + o_vc,
-                               (const int64_t *)(d_misc + 4), d_misc + 3, d_misc + 1, cap, base + o_dec,
-                               base + o_ws, ws_b, d_misc + 2, s);
-            if (st_ != ZIPVL_OK) goto done;
-            ZIPVL_CUDA(cudaMemcpyAsync(decode_out, base + o_dec, qn_b, cudaMemcpyDeviceToHost, s));
-        }
-        ZIPVL_CUDA(cudaMemcpyAsync(misc, d_misc, sizeof(misc), cudaMemcpyDeviceToHost, s));
-        if (out) ZIPVL_CUDA(cudaMemcpyAsync(out, base + o_out, qb, cudaMemcpyDeviceToHost, s));
-        if (idx_out) ZIPVL_CUDA(cudaMemcpyAsync(idx_out, base + o_idx, (size_t)a.L * 4, cudaMemcpyDeviceToHost, s));
-        ZIPVL_CUDA(cudaStreamSynchronize(s));
-        const size_t kept = (size_t)misc[0] * a.Hkv * a.D * eb;
-        if (k_cache_out) ZIPVL_CUDA(cudaMemcpyAsync(k_cache_out, base + o_kc, kept, cudaMemcpyDeviceToHost, s));
-        if (v_cache_out) ZIPVL_CUDA(cudaMemcpyAsync(v_cache_out, base + o_vc, kept, cudaMemcpyDeviceToHost, s));
-        ZIPVL_CUDA(cudaStreamSynchronize(s));
-        if (k_out) *k_out = misc[0];
-        if (misc[2] != 0)
-            st_ = fail(misc[2] & ZIPVL_DEV_TIMEOUT ? ZIPVL_ERR_TIMEOUT : ZIPVL_ERR_BAD_INDEX,
-                       "prefill_layer_host: device status word = %d", misc[2]);
-    }
-done:
-    if (base) cudaFreeAsync(base, s);
-    if (s) { cudaStreamSynchronize(s); cudaStreamDestroy(s); }
-    return st_;
 }
 
 }  // extern "C"

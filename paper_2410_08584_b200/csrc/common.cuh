@@ -132,6 +132,8 @@ cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
 // ---- launchers implemented per file -----------------------------------------
 struct LayerArgs {
     int L, Hq, Hkv, D, G;
@@ -142,7 +144,11 @@ struct LayerArgs {
     // between the sequences of Q and of K / V; per-sequence outputs are stacked likewise
     int n_seq;
     long long q_seq, kv_seq;
+    // the query heads that a launch of the tensor-core attention covers: [h0, h0 + hn), all by default
+    int h0, hn;
 };
+// api.cu: validates a layer and fills its arguments
+zipvl_status check_layer(const char *who, const zipvl_layer *l, LayerArgs *a);
 
 zipvl_status launch_score_simt(const LayerArgs &a, int dtype, const void *q, const void *k,
                                const int32_t *probe_pos, int P, float *acc, float *norm,
@@ -164,6 +170,7 @@ zipvl_status launch_compact(const LayerArgs &a, int elem_bytes, const void *k, c
                             const int32_t *idx, const int32_t *k_dev, int k_max, void *k_cache,
                             void *v_cache, int capacity, int32_t *len_out, int32_t *status_word,
                             cudaStream_t st);
+// (v == nullptr: one tensor only)
 
 // Paged cache: request b's row r lives in page table[b * stride + (r >> shift)] of a pool of
 // n_pages pages of (1 << shift) rows each.  table == nullptr: contiguous caches at cache_off.

@@ -13,6 +13,7 @@ namespace {
 constexpr int kCpThreads = 256;
 constexpr int kCpUnroll = 4;
 
+template <bool kTwo>   // K and V, or the first tensor only
 __global__ void __launch_bounds__(kCpThreads)
 compact_kernel(const uint4 *__restrict__ k, const uint4 *__restrict__ v,
                const int32_t *__restrict__ idx, const int32_t *__restrict__ k_dev, int k_max,
@@ -48,7 +49,7 @@ compact_kernel(const uint4 *__restrict__ k, const uint4 *__restrict__ v,
                 } else {
                     const long long src = (long long)t * src_row_chunks + c;
                     a[u] = __ldg(k + src);
-                    b[u] = __ldg(v + src);
+                    if (kTwo) b[u] = __ldg(v + src);
                     dst[u] = ee;
                 }
             }
@@ -57,7 +58,7 @@ compact_kernel(const uint4 *__restrict__ k, const uint4 *__restrict__ v,
         for (int u = 0; u < kCpUnroll; ++u) {
             if (dst[u] >= 0) {
                 kc[dst[u]] = a[u];
-                vc[dst[u]] = b[u];
+                if (kTwo) vc[dst[u]] = b[u];
             }
         }
     }
@@ -81,7 +82,7 @@ zipvl_status launch_compact(const LayerArgs &a, int elem_bytes, const void *k, c
     const long long cap = 148LL * 8;      // one resident wave: 8 CTAs of 256 threads per SM
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    const cudaError_t e = launch_dependent(compact_kernel, dim3((unsigned)blocks), dim3(kCpThreads), 0, st,
+    const cudaError_t e = launch_dependent(v ? compact_kernel<true> : compact_kernel<false>, dim3((unsigned)blocks), dim3(kCpThreads), 0, st,
                                            (const uint4 *)k, (const uint4 *)v, idx, k_dev, k_max, a.L,
                                            row_chunks, src_row_bytes / 16, (uint4 *)k_cache,
                                            (uint4 *)v_cache, capacity, len_out, status_word);

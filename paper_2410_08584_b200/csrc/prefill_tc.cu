@@ -155,12 +155,12 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
     }
     if (warp == 12) tmem_alloc(smem_u32(&bar->tmem_base), kTmemCols);
     grid_dependency_wait(q, k, v, idx, k_dev);   // k_dev and idx are the previous kernel's output
-    // grid.x = query head + Hq * sequence: every sequence of a batch has its own tensors, index
+    // grid.x = query head (of the launch's range) + heads * sequence: every sequence of a batch has its own tensors, index
     // list, k, output and cache, stacked; its heaviest pairs still start first
-    const int h = blockIdx.x % a.Hq, g = h / a.G;
+    const int h = a.h0 + blockIdx.x % a.hn, g = h / a.G;
     constexpr int nch = kHd >> 3;            // 16-byte chunks of a row
     {
-        const int z = blockIdx.x / a.Hq;
+        const int z = blockIdx.x / a.hn;
         q += z * a.q_seq; k += z * a.kv_seq; v += z * a.kv_seq;
         idx += (long long)z * a.L;
         k_dev += z;
@@ -173,7 +173,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
     }
     int n_valid = *k_dev;
     if (n_valid > k_max || n_valid < 0) {
-        if (h == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+        if (h == a.h0 && blockIdx.y == 0 && threadIdx.x == 0)
             report(status_word, ZIPVL_DEV_CAPACITY);
         n_valid = n_valid < 0 ? 0 : k_max;
     }
@@ -191,7 +191,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
     const int pt = n_pairs - 1 - (int)blockIdx.y;
     const int ta = pt > 0 ? 2 * pt - odd : 0;       // tile A of this CTA (tile B = ta + 1)
     const int q0 = ta * kBM;
-    const bool no_work = (pt < 0 || q0 >= n_valid || (int)blockIdx.x >= a.Hq * a.n_seq);   // or a bad grid
+    const bool no_work = (pt < 0 || q0 >= n_valid || (int)blockIdx.x >= a.hn * a.n_seq);   // or a bad grid
     const bool has_b = !(odd && pt == 0) && (q0 + kBM) < n_valid;   // tile B exists and has a valid row
     const int n_a = ta + 1;                         // key tiles of A (diagonal = ta)
     const int n_kv = has_b ? n_a + 1 : n_a;         // key tiles of B (diagonal = ta + 1)
@@ -216,7 +216,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
     const uint32_t tmem = bar->tmem_base;
     if (no_work) {                                  // a CTA past the kept set: give the columns back
         if (warp == 12) tmem_dealloc(tmem, kTmemCols);
-        if (n_valid == 0 && blockIdx.y == 0 && (int)blockIdx.x < a.Hq * a.n_seq) {
+        if (n_valid == 0 && blockIdx.y == 0 && (int)blockIdx.x < a.hn * a.n_seq) {
             // nothing kept: the results are those of the two separate calls -- an all-zero
             // PADDED output (every row is a dropped token's) and a cache of length 0
             if (out_mode == ZIPVL_OUT_PADDED) {
@@ -644,7 +644,7 @@ zipvl_status launch_prefill_tc(const LayerArgs &a, const void *q, const void *k,
     const char *env = getenv("ZIPVL_PREFILL_KERNEL");
     const int forced = !env ? 0 : (!strcmp(env, "pair") ? 1 : (!strcmp(env, "single") ? 2 : 0));
     const bool single = forced ? (forced == 2) : ((long long)k_max * a.Hq <= kSingleTileMaxRows);
-    if (single && a.n_seq == 1 && a.D == 128)
+    if (single && a.n_seq == 1 && a.D == 128 && a.hn == a.Hq)
         return launch_prefill_tc1(a, q, k, v, idx, k_dev, k_max, out, out_mode, k_cache, v_cache,
                                   capacity, len_out, status_word, st);
     auto kernel = a.half ? prefill_tc_kernel<true, 128> : prefill_tc_kernel<false, 128>;
@@ -653,7 +653,7 @@ zipvl_status launch_prefill_tc(const LayerArgs &a, const void *q, const void *k,
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess)
         return fail(ZIPVL_ERR_CUDA, "sparse_prefill: smem opt-in: %s", cudaGetErrorString(e));
-    dim3 grid(a.Hq * a.n_seq, (k_max + kPair - 1) / kPair);
+    dim3 grid(a.hn * a.n_seq, (k_max + kPair - 1) / kPair);
     e = launch_dependent(kernel, grid, dim3(kThreadsTc), kSmemBytes, st, a, (const __nv_bfloat16 *)q,
                          (const __nv_bfloat16 *)k, (const __nv_bfloat16 *)v, idx, k_dev, k_max,
                          (__nv_bfloat16 *)out, out_mode, (__nv_bfloat16 *)k_cache,
