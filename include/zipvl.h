@@ -296,13 +296,12 @@ zipvl_status zipvl_sparse_prefill_batch(const zipvl_layer *layer, const zipvl_ba
  * cache_off[b] is not a multiple of 16 bytes, is skipped as a whole (nothing of
  * its cache is read or written, its output is zeros, its length stays) and
  * reported as ZIPVL_DEV_BAD_INDEX.  The call enqueues two kernels (the second merges the cache chunks).
- * Query heads per kv head (Hq / Hkv): up to 8 for any dtype; up to 32 in 16-bit storage,
- * where grouped heads run on the tensor cores (the query heads of a kv
- * head are the rows of an MMA tile, so grouped-query attention stays bound by HBM instead of by
- * multiply-adds): one CTA per chunk of a request's cache for small problems, a persistent launch
- * (one CTA per SM over an equal share of all key/value tiles) for large ones.  Same results
- * contract on every path; ZIPVL_DECODE_KERNEL=simt|tc|tcp in the environment forces the
- * CUDA-core, the chunked or the persistent tensor-core kernel where it applies.
+ * Query heads per kv head (Hq / Hkv): up to 8 for any dtype; up to 32 in 16-bit storage.  16-bit
+ * storage runs on the tensor cores (the query heads of a kv head are the columns of an MMA, so
+ * grouped-query attention stays bound by HBM instead of by multiply-adds), but for contiguous caches
+ * of more than three requests with one query head per kv head at head_dim 64, which the CUDA-core
+ * kernel serves, as it does fp32.  Same results contract on every path; ZIPVL_DECODE_KERNEL=simt in the
+ * environment forces the CUDA-core kernel where it applies.
  */
 zipvl_status zipvl_decode(const zipvl_decode_desc *desc, const void *q, const void *k_new,
                           const void *v_new, void *k_cache, void *v_cache,
@@ -406,10 +405,8 @@ zipvl_status zipvl_decode_quant_batch(const zipvl_decode_desc *desc, const void 
  * Same arguments and results as zipvl_decode, minus ws / ws_bytes.  Limit:
  * batch * n_q_heads * ceil(max_len / chunk) * (head_dim + 2) * 4 bytes must fit
  * in 8 MiB, where chunk is the number of cache rows the library gives one thread
- * block (a power of two from 32 to 512, growing with the problem) -- e.g. batch
- * 16, 32 heads, head_dim 128 fits up to max_len 15872.  A shape the grouped-query
- * tensor-core kernels take (16-bit storage, 2 to 32 query heads per kv head) needs 4 * (ceil(max_len / chunk) + 1) such slots per query head plus
- * 4 bytes per (request, query head).  Larger problems are refused with
+ * block (from 32 to 512, growing with the problem; from 64 to 1536 for grouped query heads in 16-bit
+ * storage) -- e.g. batch 16, 32 heads, head_dim 128 fits up to max_len 15872.  Larger problems are refused with
  * ZIPVL_ERR_WORKSPACE and a message; use zipvl_decode with a workspace.
  *
  * The first call on each device looks up the array's device address (with that

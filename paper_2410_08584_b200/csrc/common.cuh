@@ -179,36 +179,22 @@ struct PageArgs {
     int stride, shift, n_pages;
 };
 
-// (Hkv and dtype decide whether the grouped-query tensor-core kernel, which leaves more partials,
-// may run: 0 / -1 = the CUDA-core layout)
+// (Hkv and dtype decide whether the grouped-query tensor-core kernel may run: 0 / -1 = it may not)
 size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv = 0, int dtype = -1);
 // workspace of the decode over the mixed-precision cache (kvquant_decode.cu)
 size_t decode_quant_ws_bytes(int B, int Hq, int Hkv, int D, int max_len);
-// caches != nullptr: the new length of request b goes to caches[b].lens[0] instead of seq_lens[b];
-// used != nullptr: used[b * (Hq / group) + hq / group] of the n_chunks slots hold a partial
-zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int chunk, int n_chunks, const float *ws,
+// caches != nullptr: the new length of request b goes to caches[b].lens[0] instead of seq_lens[b].
+zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int n_chunks, const float *ws,
                                  const int *lens, int32_t *seq_lens, void *out, cudaStream_t st,
-                                 const int *used = nullptr, int group = 1,
                                  const zipvl_quant_cache *caches = nullptr);
-// Grouped-query decode on the tensor cores: 16-bit storage, head_dim 64 / 96 / 128, 2 to 32 query
-// heads per kv head.  Two kernels that leave partials in the layout of the kernels in decode.cu and the
-// (length, appended) pairs in lens[]; the caller launches the merge.
-//   decode_tc.cu             one CTA per chunk of a (request, kv head): one partial per chunk, returns
-//                            the chunk it used (never smaller than min_chunk);
-//   decode_tc_persistent.cu  one CTA per SM over an equal share of all tiles (large batches): four
-//                            partials per CTA and (request, kv head), n_slots per (request, query
-//                            head), the number in use per (request, kv head) in used[].
-bool decode_tc_supported(const zipvl_decode_desc &d);
-zipvl_status launch_decode_tc(const zipvl_decode_desc &d, float scale_log2, const void *q,
-                              const void *k_new, const void *v_new, void *k_cache, void *v_cache,
-                              const int64_t *cache_off, PageArgs pg, const int32_t *capacity,
-                              int32_t *seq_lens, int max_len, int min_chunk, float *partials, int *lens,
-                              int32_t *status_word, cudaStream_t st, int *chunk_out);
-zipvl_status launch_decode_tcp(const zipvl_decode_desc &d, float scale_log2, const void *q,
-                               const void *k_new, const void *v_new, void *k_cache, void *v_cache,
-                               const int64_t *cache_off, PageArgs pg, const int32_t *capacity,
-                               int32_t *seq_lens, int max_len, int n_slots, float *partials, int *lens,
-                               int *used, int32_t *status_word, cudaStream_t st);
+// Decode on the tensor cores (decode_mma.cu): 16-bit storage, head_dim 64 / 96 / 128, up to
+// 32 query heads per kv head.  partials, lens: pieces of the workspace (decode.cu).
+bool decode_mma_supported(const zipvl_decode_desc &d);
+int decode_mma_chunk(int B, int Hq, int Hkv, int D, int max_len);
+zipvl_status launch_decode_mma(const zipvl_decode_desc &d, float scale_log2, const void *q, const void *k_new,
+                               const void *v_new, void *k_cache, void *v_cache, const int64_t *cache_off, PageArgs pg,
+                               const int32_t *capacity, int32_t *seq_lens, int max_len, float *partials, int *lens, void *out,
+                               int32_t *status_word, cudaStream_t st);
 zipvl_status launch_decode(const zipvl_decode_desc &d, float scale_log2, const void *q,
                            const void *k_new, const void *v_new, void *k_cache, void *v_cache,
                            const int64_t *cache_off, const int32_t *capacity, int32_t *seq_lens,

@@ -1,5 +1,7 @@
 // Decode attention over the kept cache (Algorithm 2; Eq. 4-5) for a ragged
-// batch -- an HBM stream of every cached key and value, read exactly once.
+// batch -- an HBM stream of every cached key and value, read exactly once.  This file holds the
+// CUDA-core kernel (fp32, and what dispatch_decode leaves to it), the merge kernel that all decode
+// kernels share, and the entry points; decode_mma.cu the kernel for 16-bit storage.
 //
 // Two kernels per step, the second a small programmatic dependent of the first:
 //   grid = (cache chunk, kv head x query-head tile, request).  A row of one kv
@@ -18,6 +20,8 @@
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 
@@ -282,31 +286,28 @@ __device__ __forceinline__ void store2(__nv_bfloat16 *p, float a, float b) {
 __device__ __forceinline__ void store2(__half *p, float a, float b) { *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(a, b); }
 
 // kMergeUnroll: slots per lane in flight.  8 behind the CUDA-core kernel; 6 behind the tensor-core
-// kernels, which keeps the merge at 48 registers: its CTAs then fit beside a persistent decode CTA
-// (544 threads x 96 registers) and wait there, staged, while that kernel runs.
+// kernels (48 registers: more of the merge's CTAs fit beside theirs and wait there, staged).
 template <typename T, int D, int kMergeUnroll>
 __global__ void __launch_bounds__(256, kMergeUnroll == 8 ? 4 : 5)
 decode_merge_kernel(int Hq, int lanes, int n_chunks, const float *__restrict__ ws,
                     const int *__restrict__ lens, int32_t *__restrict__ seq_lens, T *__restrict__ out,
-                    const int *__restrict__ used, int group, const zipvl_quant_cache *__restrict__ caches) {
+                    const zipvl_quant_cache *__restrict__ caches) {
     static_assert(D % 2 == 0, "two channels per thread");
     grid_launch_dependents();
-    grid_dependency_wait(ws, lens, seq_lens, used, caches);
+    grid_dependency_wait(ws, lens, seq_lens, caches);
     const int b = blockIdx.y;
     const int t = (blockIdx.x * 256 + threadIdx.x) / lanes;             // (head, channel pair) of this lane group
     const int part = threadIdx.x % lanes;
     const bool live = t < Hq * (D / 2);
     const int hq = live ? t / (D / 2) : 0, c = live ? 2 * (t % (D / 2)) : 0;
     const float *src = ws + ((long long)b * Hq + hq) * n_chunks * (D + 2);
-    // the tensor-core kernel fills only the first used[request, kv head] slots of a head
-    const int n_used = used ? min(n_chunks, max(0, used[b * (Hq / group) + hq / group])) : n_chunks;
     float M = -INFINITY, Ls = 0.f, O0 = 0.f, O1 = 0.f;
-    for (int i0 = part; i0 < n_used; i0 += kMergeUnroll * lanes) {
+    for (int i0 = part; i0 < n_chunks; i0 += kMergeUnroll * lanes) {
         float2 ml[kMergeUnroll], oi[kMergeUnroll];
 #pragma unroll
         for (int u = 0; u < kMergeUnroll; ++u) {
             const int i = i0 + u * lanes;
-            const bool in = live && i < n_used;
+            const bool in = live && i < n_chunks;
             const float *p = src + (long long)(in ? i : 0) * (D + 2);   // (a slot is (D + 2) * 4 bytes: 8-byte aligned)
             ml[u] = in ? __ldcg(reinterpret_cast<const float2 *>(p)) : make_float2(-INFINITY, 0.f);
             oi[u] = in ? __ldcg(reinterpret_cast<const float2 *>(p + 2 + c)) : make_float2(0.f, 0.f);
@@ -364,28 +365,18 @@ int decode_chunk(int B, int Hq, int max_len) {
     return c;
 }
 
-// partials per (request, query head) in the workspace: one per chunk for the CUDA-core kernel and
-// the chunked tensor-core kernel; the persistent tensor-core kernel cuts the work by tiles (a
-// request of c chunks' worth of tiles may be shared by c + 1 CTAs) and leaves four partials per CTA
-int partial_slots(int B, int Hq, int max_len, bool tc) {
-    const int chunk = decode_chunk(B, Hq, max_len);
-    const int n_chunks = (max_len + chunk - 1) / chunk;
-    return tc ? 4 * (n_chunks + 1) : n_chunks;
-}
-bool tc_shape(int Hq, int Hkv, int D, int dtype) {
+// partials in the workspace: one (m, l, o[D]) per chunk and (request, query head), for the chunking in use
+bool mma_shape(int Hq, int Hkv, int D, int dtype) {
     if (Hkv < 1 || Hq % Hkv) return false;
     const zipvl_decode_desc d = {1, Hq, Hkv, D, dtype, 0.f};
-    return decode_tc_supported(d);
+    return decode_mma_supported(d);
 }
-
-size_t partial_bytes(int B, int Hq, int D, int max_len, bool tc = false) {
-    if (tc) return ((size_t)B * Hq * partial_slots(B, Hq, max_len, true) * (D + 2) * sizeof(float) + 255) & ~(size_t)255;
-    const int chunk = decode_chunk(B, Hq, max_len);
+size_t partial_bytes(int B, int Hq, int D, int max_len, int chunk) {
     const size_t n_slots = (max_len + chunk - 1) / chunk;
     return ((size_t)B * Hq * n_slots * (D + 2) * sizeof(float) + 255) & ~(size_t)255;
 }
-// (length, appended) per request, and for the tensor-core kernel the slots in use per (request, kv head)
-size_t counter_bytes(int B, int Hq) { return (size_t)(2 * B + B * Hq) * sizeof(int); }
+// (length, appended) per request
+size_t length_bytes(int B) { return (size_t)2 * B * sizeof(int); }
 
 template <typename T, int D>
 zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, const void *k_new,
@@ -396,7 +387,7 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
     const int chunk = decode_chunk(B, Hq, max_len);
     const int n_chunks = (max_len + chunk - 1) / chunk;
     float *wsf = reinterpret_cast<float *>(ws);
-    int *lens = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + partial_bytes(B, Hq, D, max_len));
+    int *lens = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + partial_bytes(B, Hq, D, max_len, chunk));
 #define ZIPVL_DEC_P(GT_, P_)                                                                    \
     {                                                                                           \
         dim3 grid(n_chunks, Hkv * ((G + GT_ - 1) / GT_), B);                                    \
@@ -421,7 +412,7 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
         const int lanes = merge_lanes(B, Hq, D, n_chunks);
         le = launch_dependent(decode_merge_kernel<T, D, 8>, merge_grid(B, Hq, D, lanes), dim3(256), 0, st, Hq,
                               lanes, n_chunks, (const float *)wsf, (const int *)lens, seq_lens, (T *)out,
-                              (const int *)nullptr, 1, (const zipvl_quant_cache *)nullptr);
+                              (const zipvl_quant_cache *)nullptr);
     }
     if (le != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "zipvl_decode: launch: %s", cudaGetErrorString(le));
     count_launches(2);
@@ -432,15 +423,14 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
 
 // what the tensor-core kernels and the decode over a quantised cache (kvquant_decode.cu) share with
 // this file: the layout of the partial results and the merge kernel
-zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int chunk, int n_chunks, const float *ws,
+zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int n_chunks, const float *ws,
                                  const int *lens, int32_t *seq_lens, void *out, cudaStream_t st,
-                                 const int *used, int group, const zipvl_quant_cache *caches) {
+                                 const zipvl_quant_cache *caches) {
     cudaError_t le = cudaErrorInvalidValue;
-    (void)chunk;
     const int lanes = merge_lanes(B, Hq, D, n_chunks);
     const dim3 grid = merge_grid(B, Hq, D, lanes);
 #define ZIPVL_MERGE(T_, D_) \
-    le = launch_dependent(decode_merge_kernel<T_, D_, 6>, grid, dim3(256), 0, st, Hq, lanes, n_chunks, ws, lens, seq_lens, (T_ *)out, used, group, caches)
+    le = launch_dependent(decode_merge_kernel<T_, D_, 6>, grid, dim3(256), 0, st, Hq, lanes, n_chunks, ws, lens, seq_lens, (T_ *)out, caches)
     if (dtype == ZIPVL_BF16 && D == 128) ZIPVL_MERGE(__nv_bfloat16, 128);
     else if (dtype == ZIPVL_BF16 && D == 96) ZIPVL_MERGE(__nv_bfloat16, 96);
     else if (dtype == ZIPVL_BF16 && D == 64) ZIPVL_MERGE(__nv_bfloat16, 64);
@@ -454,7 +444,10 @@ zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int chunk, int
 }
 
 size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv, int dtype) {
-    return partial_bytes(B, Hq, D, max_len, tc_shape(Hq, Hkv, D, dtype)) + counter_bytes(B, Hq);
+    // (a shape of the tensor-core kernel may be sent to the CUDA-core one, see dispatch_decode)
+    const size_t simt = partial_bytes(B, Hq, D, max_len, decode_chunk(B, Hq, max_len));
+    const size_t mma = mma_shape(Hq, Hkv, D, dtype) ? partial_bytes(B, Hq, D, max_len, decode_mma_chunk(B, Hq, Hkv, D, max_len)) : 0;
+    return std::max(simt, mma) + length_bytes(B);
 }
 
 namespace {
@@ -463,47 +456,26 @@ zipvl_status dispatch_decode(const zipvl_decode_desc &d, float scale_log2, const
                              const int64_t *cache_off, PageArgs pg, const int32_t *capacity,
                              int32_t *seq_lens, int max_len, void *out, void *ws,
                              int32_t *status_word, cudaStream_t st) {
-    // Grouped-query attention in 16-bit storage runs on the tensor cores from two query heads per
-    // kv head on: there the CUDA-core kernel is bound by its multiply-adds (0.49 of the HBM copy
-    // rate at four heads per kv head, 0.29 at seven; at two it reaches 0.81 against 0.84).  Of the
-    // two tensor-core kernels the persistent one takes the large problems (from about ten
-    // key/value tiles per SM on it is 5 to 15 % faster: no CTA prologue between work items); below
-    // that the launch of one CTA per chunk is quicker (fewer partials to merge, shorter CTAs).
-    // ZIPVL_DECODE_KERNEL=simt|tc|tcp overrides the choice (measurements, tests).
-    {
-        const char *env = getenv("ZIPVL_DECODE_KERNEL");
-        const int G = d.n_q_heads / d.n_kv_heads;
-        const long long tiles = (long long)d.batch * d.n_kv_heads * ((max_len + 127) / 128);
-        constexpr long long kPersistentFrom = 1500;
-        const bool want_simt = env && !strcmp(env, "simt");
-        if (decode_tc_supported(d) && (!want_simt || G > 8)) {
-            const int B = d.batch, Hq = d.n_q_heads, D = d.head_dim;
-            const bool persistent = env && !strcmp(env, "tcp") ? true
-                                    : (env && !strcmp(env, "tc") ? false : tiles >= kPersistentFrom);
-            float *wsf = reinterpret_cast<float *>(ws);
-            int *lens = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + partial_bytes(B, Hq, D, max_len, true));
-            int *used = lens + 2 * B;
-            int chunk = decode_chunk(B, Hq, max_len);
-            zipvl_status sm;
-            if (persistent) {
-                const int n_slots = partial_slots(B, Hq, max_len, true);    // as the workspace was sized
-                const zipvl_status s = launch_decode_tcp(d, scale_log2, q, k_new, v_new, k_cache, v_cache,
-                                                         cache_off, pg, capacity, seq_lens, max_len, n_slots, wsf,
-                                                         lens, used, status_word, st);
-                if (s != ZIPVL_OK) return s;
-                sm = launch_decode_merge(d.dtype, D, Hq, B, chunk, n_slots, wsf, lens, seq_lens, out, st, used, G);
-            } else {
-                const zipvl_status s = launch_decode_tc(d, scale_log2, q, k_new, v_new, k_cache, v_cache, cache_off,
-                                                        pg, capacity, seq_lens, max_len, chunk, wsf, lens,
-                                                        status_word, st, &chunk);
-                if (s != ZIPVL_OK) return s;
-                sm = launch_decode_merge(d.dtype, D, Hq, B, chunk, (max_len + chunk - 1) / chunk, wsf, lens,
-                                         seq_lens, out, st);
-            }
-            return sm != ZIPVL_OK ? sm : check_launch("zipvl_decode");
-        }
-        if (G > 8) return fail(ZIPVL_ERR_UNSUPPORTED, "decode: %d query heads per kv head", G);
+    // 16-bit storage runs on the tensor cores: with several query heads per row the CUDA-core
+    // kernel is bound by its multiply-adds (0.49 of the HBM copy rate at four, 0.29 at seven) and
+    // reads a row once per eight heads; with one it has too few rows in flight on short caches
+    // (one request of 2307 rows: 13.8 against 11.2 us) and too much address arithmetic on
+    // paged ones (26 requests of 560 rows: 57 against 44 us).  It keeps the contiguous caches of many requests
+    // at head_dim 64 (37 requests of 1.3K-3.1K rows: 61 against 64 us).
+    // ZIPVL_DECODE_KERNEL=simt in the environment sends shapes of up to eight heads to the CUDA-core kernel
+    // all the same (measurements, tests).
+    const char *env = getenv("ZIPVL_DECODE_KERNEL");
+    const int Hq = d.n_q_heads, Hkv = d.n_kv_heads;
+    const bool simt = Hq / Hkv <= 8 && ((env && !strcmp(env, "simt")) ||
+                                        (Hq == Hkv && d.head_dim == 64 && !pg.table && d.batch > 3));
+    if (decode_mma_supported(d) && !simt) {
+        const int chunk = decode_mma_chunk(d.batch, Hq, Hkv, d.head_dim, max_len);
+        int *lens = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + partial_bytes(d.batch, Hq, d.head_dim, max_len, chunk));
+        const zipvl_status s = launch_decode_mma(d, scale_log2, q, k_new, v_new, k_cache, v_cache, cache_off, pg, capacity,
+                                                 seq_lens, max_len, reinterpret_cast<float *>(ws), lens, out, status_word, st);
+        return s != ZIPVL_OK ? s : check_launch("zipvl_decode");
     }
+    if (Hq / Hkv > 8) return fail(ZIPVL_ERR_UNSUPPORTED, "decode: %d query heads per kv head", Hq / Hkv);
 #define ZIPVL_ARGS d, scale_log2, q, k_new, v_new, k_cache, v_cache, cache_off, pg, capacity, \
                    seq_lens, max_len, out, ws, status_word, st
     if (d.dtype == ZIPVL_BF16) {
@@ -582,7 +554,7 @@ extern "C" zipvl_status zipvl_decode_noalloc(const zipvl_decode_desc *d, const v
                     d->n_q_heads, d->n_kv_heads);
     if ((d->dtype != ZIPVL_BF16 && d->dtype != ZIPVL_F32 && d->dtype != ZIPVL_F16) ||
         (d->head_dim != 64 && d->head_dim != 96 && d->head_dim != 128) ||
-        (d->n_q_heads / d->n_kv_heads > 8 && !decode_tc_supported(*d)))
+        (d->n_q_heads / d->n_kv_heads > 8 && !decode_mma_supported(*d)))
         return fail(ZIPVL_ERR_UNSUPPORTED, "%s: dtype %d head_dim %d group %d", who, d->dtype,
                     d->head_dim, d->n_q_heads / d->n_kv_heads);
     if (!q || !k_cache || !v_cache || !cache_off || !capacity || !seq_lens || !out)
@@ -626,7 +598,7 @@ extern "C" zipvl_status zipvl_decode_paged(const zipvl_decode_desc *d, const voi
                     d->n_q_heads, d->n_kv_heads);
     if ((d->dtype != ZIPVL_BF16 && d->dtype != ZIPVL_F32 && d->dtype != ZIPVL_F16) ||
         (d->head_dim != 64 && d->head_dim != 96 && d->head_dim != 128) ||
-        (d->n_q_heads / d->n_kv_heads > 8 && !decode_tc_supported(*d)))
+        (d->n_q_heads / d->n_kv_heads > 8 && !decode_mma_supported(*d)))
         return fail(ZIPVL_ERR_UNSUPPORTED, "%s: dtype %d head_dim %d group %d", who, d->dtype,
                     d->head_dim, d->n_q_heads / d->n_kv_heads);
     if (!q || !k_pages || !v_pages || !block_table || !capacity || !seq_lens || !out || !ws)

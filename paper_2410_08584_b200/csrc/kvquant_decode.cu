@@ -493,7 +493,7 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
                                            lens_ws, status_word);
     if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "zipvl_decode_quant: launch: %s", cudaGetErrorString(e));
     count_launches(1);
-    return launch_decode_merge(d.dtype, D, Hq, B, chunk, n_chunks, wsf, lens_ws, lens, out, st, nullptr, 1, caches);
+    return launch_decode_merge(d.dtype, D, Hq, B, n_chunks, wsf, lens_ws, lens, out, st, caches);
 }
 
 }  // namespace
