@@ -652,12 +652,42 @@ __device__ __forceinline__ unsigned long long solo_sum(const SoloSmem &sm, int b
 struct SoloCtl {                       // static shared memory
     unsigned long long wsum[kSoloWarps], sum_gt, bin_sum;
     unsigned int wcnt[kSoloWarps], wmin[2][kSoloWarps], wmax[2][kSoloWarps];
-    unsigned int hit, hit_bin, cnt_gt, bin_cnt, one_key;
+    unsigned int hit, hit_bin, cnt_gt, bin_cnt, one_key, need;
     // the tokens of a sparsely filled crossing bin, resolved by one warp (see kDirect)
     unsigned int n_cand, cand_key[32];
     unsigned long long cand_fx[32];
 };
 constexpr unsigned int kDirect = 32;   // a crossing bin with this many tokens or fewer skips the next level
+
+// sum over the warp, the operand below 2^60 / 32: three 20-bit pieces, one instruction each
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
+    return (unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned int)v & 0xfffffu) +
+           ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned int)(v >> 20) & 0xfffffu) << 20) +
+           ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned int)(v >> 40)) << 40);
+}
+
+// block-wide exclusive prefix, in thread order, of two counts below 2^16 in one word, and the total
+__device__ __forceinline__ unsigned int solo_scan2(unsigned int v, SoloCtl &c, unsigned int *total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned int inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    __syncthreads();                                   // earlier readers of wcnt are done
+    if (lane == 31) c.wcnt[w] = inc;
+    __syncthreads();
+    unsigned int before = 0, all = 0;
+#pragma unroll
+    for (int i = 0; i < kSoloWarps; ++i) {
+        const unsigned int x = c.wcnt[i];
+        if (i < w) before += x;
+        all += x;
+    }
+    *total = all;
+    return before + inc - v;
+}
 
 // block-wide (256 threads) exclusive prefix of a (count, sum) pair in thread order, and totals
 __device__ __forceinline__ void solo_scan(unsigned int vc, unsigned long long vs, SoloCtl &c,
@@ -707,7 +737,7 @@ __device__ __forceinline__ bool solo_bin(unsigned int key, unsigned int base, in
 // the fine search: (1) every warp adds up its bins (kBins / warps, from the top), (2) warp 0
 // walks the warp totals to the warp where the running total crosses, (3) that warp scans its
 // lanes and the lane that crosses walks its own bins.
-__device__ void solo_find_bin(const SoloSmem &sm, bool by_sum, unsigned long long target,
+__device__ void solo_find_bin(const SoloSmem &sm, const unsigned int *cnt, bool by_sum, unsigned long long target,
                               unsigned int carry_cnt, unsigned long long carry_sum, SoloCtl &c) {
     constexpr int kPer = kBins / kSoloThreads;         // bins per thread
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -716,7 +746,7 @@ __device__ void solo_find_bin(const SoloSmem &sm, bool by_sum, unsigned long lon
     unsigned int lc = 0;
 #pragma unroll
     for (int v4 = 0; v4 < kPer / 4; ++v4) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(&sm.cnt[b_top - 3 - 4 * v4]);
+        const uint4 q = *reinterpret_cast<const uint4 *>(&cnt[b_top - 3 - 4 * v4]);
         cb[4 * v4 + 0] = q.w; cb[4 * v4 + 1] = q.z; cb[4 * v4 + 2] = q.y; cb[4 * v4 + 3] = q.x;
         lc += q.x + q.y + q.z + q.w;
     }
@@ -730,9 +760,7 @@ __device__ void solo_find_bin(const SoloSmem &sm, bool by_sum, unsigned long lon
     const unsigned int wc = __reduce_add_sync(0xffffffffu, lc);
     unsigned long long wsum = 0;
     if (by_sum) {
-        wsum = (unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned int)ls & 0xfffffu) +
-               ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned int)(ls >> 20) & 0xfffffu) << 20) +
-               ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned int)(ls >> 40)) << 40);
+        wsum = warp_sum64(ls);
     }
     __syncthreads();                                   // earlier readers of wcnt / wsum / hit are done
     if (lane == 0) { c.wcnt[w] = wc; c.wsum[w] = wsum; }
@@ -858,6 +886,10 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
         mx[x] = __reduce_max_sync(0xffffffffu, mx[x]);
         if (lane == 0) { c.wmin[x][warp] = mn[x]; c.wmax[x][warp] = mx[x]; }
     }
+    {
+        const unsigned long long ws = warp_sum64(my_sum);
+        if (lane == 0) c.wsum[warp] = ws;
+    }
     __syncthreads();                   // the ranges are in; the histograms are clear
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
@@ -865,6 +897,9 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
 #pragma unroll
         for (int i = 0; i < kSoloWarps; ++i) { mn[x] = min(mn[x], c.wmin[x][i]); mx[x] = max(mx[x], c.wmax[x][i]); }
     }
+    unsigned long long S_b = 0;
+#pragma unroll
+    for (int i = 0; i < kSoloWarps; ++i) S_b += c.wsum[i];
     auto first_shift = [](unsigned int lo, unsigned int hi) {
         const int bits = 32 - __clz(hi - lo);          // bits of the span (0 when all keys are equal)
         return bits > 12 ? bits - 12 : 0;
@@ -889,22 +924,11 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
         if (!by_sum && p >= (unsigned int)L) break;
         const unsigned int *keys = by_sum ? kb : kr;
         unsigned long long target = p;
-        if (by_sum) {
-            unsigned int uc;
-            unsigned long long us, S_b;
-            solo_scan(0u, my_sum, c, &uc, &us, nullptr, &S_b);
-            target = (unsigned long long)ceil((double)tau * (double)S_b);
-        }
+        if (by_sum) target = (unsigned long long)ceil((double)tau * (double)S_b);
         unsigned int base = mn[pass], carry_c = 0;
         unsigned long long carry_s = 0;
         int shift = shift1[pass], width_log2 = 32;
         bool found = true;
-        if (!by_sum) {
-            // the ranking level 1 was counted into cnt_r: bring it to where the search reads
-            __syncthreads();
-            for (int e = threadIdx.x; e < kBins / 4; e += kSoloThreads)
-                reinterpret_cast<uint4 *>(sm.cnt)[e] = reinterpret_cast<const uint4 *>(sm.cnt_r)[e];
-        }
 #pragma unroll 1
         for (int level = 0;; ++level) {
             if (level > 0) {
@@ -923,7 +947,8 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
                 }
             }
             __syncthreads();
-            solo_find_bin(sm, by_sum, target, carry_c, carry_s, c);
+            // (the ranking level 1 was counted into cnt_r)
+            solo_find_bin(sm, !by_sum && level == 0 ? sm.cnt_r : sm.cnt, by_sum, target, carry_c, carry_s, c);
             if (c.hit == 0xffffffffu) { found = false; break; }     // (rounding let no prefix qualify)
             if (shift == 0) { thr_key = base + c.hit_bin; break; }  // the bin is one key value
             if (c.bin_cnt <= kDirect) {
@@ -987,13 +1012,18 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
         }
         if (by_sum) {
             if (found) {
-                // copies of the threshold value enter one at a time
-                const unsigned long long v = c.bin_cnt ? c.bin_sum / c.bin_cnt : 0ull;
-                unsigned long long need = 1;
-                if (target > c.sum_gt && v > 0) need = (target - c.sum_gt + v - 1) / v;
-                if (need < 1) need = 1;
-                if (need > c.bin_cnt) need = c.bin_cnt;
-                p = c.cnt_gt + (unsigned int)need;
+                // copies of the threshold value enter one at a time (one thread divides: a 64-bit
+                // division by every thread of the CTA takes a microsecond)
+                if (c.bin_cnt > 1) {
+                    if (threadIdx.x == 0) {
+                        const unsigned long long v = c.bin_sum / c.bin_cnt;
+                        unsigned long long need = 1;
+                        if (target > c.sum_gt && v > 0) need = (target - c.sum_gt + v - 1) / v;
+                        c.need = (unsigned int)(need < 1 ? 1 : need > c.bin_cnt ? c.bin_cnt : need);
+                    }
+                    __syncthreads();
+                }
+                p = c.cnt_gt + (c.bin_cnt > 1 ? c.need : c.bin_cnt);
             }
             thr_key = 0;
         } else {
@@ -1012,11 +1042,11 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
             n_eq += kr[e] == thr_key;
         }
     }
-    unsigned int eq_before;
-    unsigned long long gt_before;
-    solo_scan(n_eq, (unsigned long long)n_gt, c, &eq_before, &gt_before);
+    unsigned int total2;
+    const unsigned int before2 = solo_scan2(n_gt | (n_eq << 16), c, &total2);
+    const unsigned int gt_before = before2 & 0xffffu, eq_before = before2 >> 16;
     const unsigned int eq_take = all_sel ? n_eq : min(n_eq, need_eq > eq_before ? need_eq - eq_before : 0u);
-    unsigned int out = all_sel ? (unsigned int)min(j0, L) : (unsigned int)gt_before + min(eq_before, need_eq);
+    unsigned int out = all_sel ? (unsigned int)min(j0, L) : gt_before + min(eq_before, need_eq);
     unsigned int tot_sel = all_sel ? (unsigned int)L : p;
     const unsigned int keep_last = mode >> 8;
     const int f0 = (kKeepLast && keep_last > 0 && !all_sel) ? max(0, L - (int)min(keep_last, (unsigned int)L)) : L;
@@ -1049,12 +1079,12 @@ select_solo_kernel(int L, const float *__restrict__ acc, const float *__restrict
                 if (!keep && kr[e] == thr_key && eq_left > 0) { keep = true; --eq_left; }
                 if (kKeepLast) keep = keep || (j >= f0);
             }
-            const unsigned long long fx = to_fx(av[e]);
-            all += fx;
-            if (keep) {
-                idx[out++] = j;
-                mass += fx;
+            if (kept_mass) {
+                const unsigned long long fx = to_fx(av[e]);
+                all += fx;
+                if (keep) mass += fx;
             }
+            if (keep) idx[out++] = j;
         }
     }
     for (int j = tot_sel + threadIdx.x; j < L; j += kSoloThreads) idx[j] = -1;
@@ -1272,10 +1302,14 @@ select_cluster_kernel(int L, const float *__restrict__ acc, const float *__restr
         if (lane == 0) { c.wmin[x][warp] = mn[x]; c.wmax[x][warp] = mx[x]; }
     }
     {
-        unsigned int uc;
-        unsigned long long us, S;
-        solo_scan(0u, my_sum, c, &uc, &us, nullptr, &S);
+        const unsigned long long ws = warp_sum64(my_sum);
+        if (lane == 0) c.wsum[warp] = ws;
+    }
+    __syncthreads();
+    {
         if (threadIdx.x == 0) {
+            unsigned long long S = 0;
+            for (int i = 0; i < kSoloWarps; ++i) S += c.wsum[i];
             sm.sum = S;
             for (int x = 0; x < 2; ++x) {
                 unsigned int lo = 0xffffffffu, hi = 0u;
@@ -1448,13 +1482,18 @@ select_cluster_kernel(int L, const float *__restrict__ acc, const float *__restr
         }
         if (by_sum) {
             if (found) {
-                // copies of the threshold value enter one at a time
-                const unsigned long long v = c.bin_cnt ? c.bin_sum / c.bin_cnt : 0ull;
-                unsigned long long need = 1;
-                if (target > c.sum_gt && v > 0) need = (target - c.sum_gt + v - 1) / v;
-                if (need < 1) need = 1;
-                if (need > c.bin_cnt) need = c.bin_cnt;
-                p = c.cnt_gt + (unsigned int)need;
+                // copies of the threshold value enter one at a time (one thread divides: a 64-bit
+                // division by every thread of the CTA takes a microsecond)
+                if (c.bin_cnt > 1) {
+                    if (threadIdx.x == 0) {
+                        const unsigned long long v = c.bin_sum / c.bin_cnt;
+                        unsigned long long need = 1;
+                        if (target > c.sum_gt && v > 0) need = (target - c.sum_gt + v - 1) / v;
+                        c.need = (unsigned int)(need < 1 ? 1 : need > c.bin_cnt ? c.bin_cnt : need);
+                    }
+                    __syncthreads();
+                }
+                p = c.cnt_gt + (c.bin_cnt > 1 ? c.need : c.bin_cnt);
             }
             thr_key = 0;
             __syncthreads();           // (c is rewritten by the next search)
@@ -1473,13 +1512,13 @@ select_cluster_kernel(int L, const float *__restrict__ acc, const float *__restr
             n_eq += kr[e] == thr_key;
         }
     }
-    unsigned int eq_before, eq_here;
-    unsigned long long gt_before, gt_here;
-    solo_scan(n_eq, (unsigned long long)n_gt, c, &eq_before, &gt_before, &eq_here, &gt_here);
+    unsigned int here2;                // (a CTA has at most 8192 tokens)
+    const unsigned int before2 = solo_scan2(n_gt | (n_eq << 16), c, &here2);
+    unsigned int gt_before = before2 & 0xffffu, eq_before = before2 >> 16;
     if (!all_sel) {
         // what the CTAs in front hold
         if (!counted) {
-            if (threadIdx.x == 0) { sm.n_gt = (unsigned int)gt_here; sm.n_eq = eq_here; }
+            if (threadIdx.x == 0) { sm.n_gt = here2 & 0xffffu; sm.n_eq = here2 >> 16; }
             cl.sync();
         }
         unsigned int g = 0, q = 0;
@@ -1501,7 +1540,7 @@ select_cluster_kernel(int L, const float *__restrict__ acc, const float *__restr
         eq_before += __reduce_add_sync(0xffffffffu, q);
     }
     const unsigned int eq_take = all_sel ? n_eq : min(n_eq, need_eq > eq_before ? need_eq - eq_before : 0u);
-    unsigned int out = all_sel ? (unsigned int)min(j0, j_end) : (unsigned int)gt_before + min(eq_before, need_eq);
+    unsigned int out = all_sel ? (unsigned int)min(j0, j_end) : gt_before + min(eq_before, need_eq);
     unsigned int tot_sel = all_sel ? (unsigned int)L : p;
     const unsigned int keep_last = mode >> 8;
     const int f0 = (kKeepLast && keep_last > 0 && !all_sel) ? max(0, L - (int)min(keep_last, (unsigned int)L)) : L;
