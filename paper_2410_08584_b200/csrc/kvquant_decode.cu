@@ -380,7 +380,7 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *ring = smem + (threadIdx.x >> 5) * Ring<D>::kBytes;
     const int b = blockIdx.z, lane = threadIdx.x & 31;
-    const int hkv = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    const int hkv = blockIdx.y * kWarps + (threadIdx.x >> 5);
     const bool first = blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0;
     const bool blocks_ok = request_blocks(caches, b, qb, lens);
     const int old_hi = blocks_ok ? lens[0] : 0, n_lo = blocks_ok ? lens[1] : 0;
@@ -402,15 +402,15 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
         lens_ws[2 * b + 1] = room ? 1 : 0;
     }
     if (hkv >= Hkv) return;
-    const int c0 = blockIdx.y * chunk, c1 = min(total, c0 + chunk);
-    float *dst = ws + (((long long)b * Hq + hkv * G) * n_chunks + blockIdx.y) * (D + 2);
+    const int c0 = blockIdx.x * chunk, c1 = min(total, c0 + chunk);
+    float *dst = ws + (((long long)b * Hq + hkv * G) * n_chunks + blockIdx.x) * (D + 2);
     const long long head_pitch = (long long)n_chunks * (D + 2);
     // the appended row belongs to the chunk that ends with it (or, beyond the rows that count, to the last)
     const long long rh = (long long)old_hi * Hkv + hkv;
     NewRow fresh = {k_new + ((long long)b * Hkv + hkv) * D, v_new + ((long long)b * Hkv + hkv) * D, qb.k_hi + rh * (D / 2),
                     qb.v_hi + rh * (D / 2), qb.p_hi + rh * 4};
     const bool mine = room && old_hi >= c0 && old_hi < c1;
-    if (room && old_hi >= total && (int)blockIdx.y == n_chunks - 1) {
+    if (room && old_hi >= total && (int)blockIdx.x == n_chunks - 1) {
         uint32_t par;
         fresh.quantise<kHalf, D>(lane, par);
     }
@@ -487,7 +487,7 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
     constexpr int smem = kWarps * Ring<D>::kBytes;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "zipvl_decode_quant: smem opt-in: %s", cudaGetErrorString(e));
-    e = launch_dependent(kernel, dim3((Hkv + kWarps - 1) / kWarps, n_chunks, B), dim3(kWarps * 32), smem, st,
+    e = launch_dependent(kernel, dim3(n_chunks, (Hkv + kWarps - 1) / kWarps, B), dim3(kWarps * 32), smem, st,
                                            Hq, Hkv, scale_log2, (const unsigned short *)q, (const unsigned short *)k_new,
                                            (const unsigned short *)v_new, qb, lens, caches, max_len, chunk, n_chunks, wsf,
                                            lens_ws, status_word);

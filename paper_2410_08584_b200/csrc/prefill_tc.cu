@@ -256,7 +256,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
         // (The query rows are gathered by the softmax warps at the same time.)
         int issued = 0;
         for (int seq = 0; seq < total; ++seq) {
-            while (issued < total && issued - seq < (seq == 0 ? 1 : kWindow) && slot_free(issued, issued == seq))
+            while (issued < total && issued - seq < kWindow && slot_free(issued, issued == seq))
                 issue(issued++);
             const int newer = issued - 1 - seq;     // groups younger than `seq` in flight
             if (newer >= 2) cp_async_wait<2>();

@@ -100,8 +100,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, LayerArgs a,
     const int t1 = min(n_tiles_all, t0 + tiles_per_chunk);
     const int n_tiles = t1 - t0;
     if (n_tiles <= 0) return;
-    // <1> walks its tiles backwards: where K outgrows L2, the tiles that <0> read last are still there
-    auto tile_of = [&](int n) { return MODE == 0 ? t0 + n : t1 - 1 - n; };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -156,7 +154,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, LayerArgs a,
                 // row, where the copy fills zeros; no MMA reads those columns)
                 mbar_expect_tx(fb, kHd > 64 ? kTileBytes : kHalfBytes);
                 const uint32_t dst = sK + s * kTileBytes;
-                const int y = z * a.L + tile_of(n) * kTile;
+                const int y = z * a.L + (t0 + n) * kTile;
                 tma_load_2d(dst, &kmap, g * kHd, y, fb);
                 if (kHd > 64) tma_load_2d(dst + kHalfBytes, &kmap, g * kHd + 64, y, fb);
             }
@@ -236,7 +234,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, LayerArgs a,
         float m = -INFINITY, l = 0.f;
         for (int n = 0; n < n_tiles; ++n) {
             const int b = n & 1;
-            const int j0 = tile_of(n) * kTile;
+            const int j0 = (t0 + n) * kTile;
             mbar_wait(smem_u32(&bar->s_full[b]), (n >> 1) & 1, abort_flag);
             tc_fence_after();
             const uint32_t tS = lane_base + b * 128;
