@@ -256,7 +256,9 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
         // (The query rows are gathered by the softmax warps at the same time.)
         int issued = 0;
         for (int seq = 0; seq < total; ++seq) {
-            while (issued < total && issued - seq < kWindow && slot_free(issued, issued == seq))
+            // The first K tile goes alone: a cold CTA waits for its queries and that tile, and the copies behind
+            // it would only share the memory (2944 tokens, 32 heads, whole layer: 103.5 -> 102.3 us).
+            while (issued < total && issued - seq < (seq == 0 ? 1 : kWindow) && slot_free(issued, issued == seq))
                 issue(issued++);
             const int newer = issued - 1 - seq;     // groups younger than `seq` in flight
             if (newer >= 2) cp_async_wait<2>();
