@@ -721,7 +721,7 @@ def decode_benchmark(z, dev, steps, peaks, B=16, ctx_max=32768):
 
 def decode_gqa_benchmark(z, dev, peaks, steps=64, B=16, Hq=28, Hkv=4, d=128, len_max=30000):
     """Grouped-query decode (the long-video model's head shape: 28 query heads on 4 kv heads) on kept
-    caches of 6K-30K rows: the tensor-core kernel (default from three query heads per kv head) next to
+    caches of 6K-30K rows: the tensor-core kernel (the library's choice) next to
     the CUDA-core kernel, which ZIPVL_DECODE_KERNEL selects; one request checked against the oracle."""
     import oracle
     g = torch.Generator().manual_seed(BASE_SEED + 6)
@@ -746,8 +746,7 @@ def decode_gqa_benchmark(z, dev, peaks, steps=64, B=16, Hq=28, Hkv=4, d=128, len
     prev = os.environ.get("ZIPVL_DECODE_KERNEL")
     try:
         for name in ("tensor_core", "cuda_core"):
-            # the library's own choice of tensor-core kernel (chunked or persistent, by problem size)
-            # against the CUDA-core kernel forced
+            # the library's own choice, the tensor-core kernel, against the CUDA-core kernel forced
             if name == "tensor_core":
                 os.environ.pop("ZIPVL_DECODE_KERNEL", None)
             else:

@@ -153,7 +153,7 @@ zipvl_status zipvl_score(const zipvl_layer *layer, const void *q, const void *k,
  * that the scores sum to n); fixed_k > 0 replaces the adaptive p (fixed-ratio
  * ablation, Table 3) and is clamped to L.  Sums are taken in 2^-34 fixed point,
  * so results do not depend on thread order and repeat bit for bit.  The call
- * enqueues one kernel, preceded for rows longer than 4096 tokens by one memset
+ * enqueues one kernel, preceded for rows longer than 65536 tokens by one memset
  * of its workspace.  mode: ZIPVL_BUDGET_BY_NORM, ZIPVL_TOPK_BY_ACC, ZIPVL_KEEP_LAST(r) or'ed
  * together; any other bit is ZIPVL_ERR_INVALID_ARG.
  *
@@ -352,7 +352,7 @@ zipvl_status zipvl_decode_paged(const zipvl_decode_desc *desc, const void *q, co
  * append); out[h,:] = softmax attention of q[h,:] over all dequantised rows.  max_len: host
  * bound on lens[0] + lens[1] after the append; ws: zipvl_workspace_bytes(ZIPVL_OP_DECODE) for
  * batch 1 and L = max_len.  16-bit storage types, head_dim 64 or 128, 1, 2 or 4 query heads per
- * KV head, at most 64 KV heads.  The call enqueues two kernels (three with an append).
+ * KV head, at most 64 KV heads.  The call enqueues two kernels, with or without an append.
  */
 zipvl_status zipvl_quantize_kv(const zipvl_layer *layer, const void *k, const void *v, const int32_t *idx,
                                const int32_t *k_dev, int32_t k_max, void *k_hi, void *v_hi,
@@ -375,7 +375,7 @@ zipvl_status zipvl_decode_quant(const zipvl_decode_desc *desc, const void *q, co
  * there: a request whose entry has a NULL or misaligned block, or a capacity below 1, is
  * skipped (nothing appended, an output of zeros) and reported as ZIPVL_DEV_BAD_INDEX; a full
  * 4-bit block as ZIPVL_DEV_CAPACITY, per request.  Same shapes as zipvl_decode_quant.
- * The call enqueues two kernels (three with an append), whatever the batch.
+ * The call enqueues two kernels, whatever the batch and with or without an append.
  */
 typedef struct zipvl_quant_cache {
     void *k_hi, *v_hi, *params_hi;   /* the 4-bit block */
@@ -455,8 +455,8 @@ zipvl_status zipvl_layer_step_host(const zipvl_layer *layer, const void *q, cons
                                    const void *k_new, const void *v_new, void *decode_out);
 
 /*
- * zipvl_release_host_scratch -- give back the device memory zipvl_prefill_layer_host
- * keeps between calls.  (No counterpart in the paper.)  That call takes its device
+ * zipvl_release_host_scratch -- give back the device memory, streams and events zipvl_prefill_layer_host
+ * and zipvl_layer_step_host keep between calls.  (No counterpart in the paper.)  That call takes its device
  * scratch from a memory pool of the library's own, one per device, which keeps freed
  * memory for the next call instead of returning it to the driver; this function trims
  * the current device's pool to zero.  Safe to call at any time; a no-op if

@@ -380,7 +380,9 @@ int decode_mma_chunk(int B, int Hq, int Hkv, int D, int max_len) {
     const int nt = Hq == Hkv ? 0 : (Hq / Hkv + 7) / 8;
     const long long groups = (long long)B * Hkv, wave = 148 * ctas_per_sm(nt, D);
     const int n = (int)std::max(1ll, wave / groups);
-    return std::min(max_rows(Hq / Hkv, D), std::max(64, ((max_len + n - 1) / n + 63) / 64 * 64));
+    const auto tiles_of = [&](long long parts) { return (int)((max_len + parts - 1) / parts + 63) / 64 * 64; };
+    // (the last term: chunks are the grid's y, which ends at 65535)
+    return std::max(std::min(max_rows(Hq / Hkv, D), std::max(64, tiles_of(n))), tiles_of(65535));
 }
 
 zipvl_status launch_decode_mma(const zipvl_decode_desc &d, float scale_log2, const void *q, const void *k_new,
