@@ -21,8 +21,8 @@
 //   warp 12    issues tcgen05.mma: S_X = Q_X K^T (shared-memory operands) and
 //              O_X += P_X V (P from tensor memory, V as MN-major operand), the two
 //              query tiles interleaved so the tensor pipe works on one while the
-//              other is in softmax.  It looks at its barriers in turn and serves
-//              whichever tile is ready.
+//              other is in softmax.  The tiles take turns and it sleeps on the barrier of
+//              the one that comes next.
 //   warps 13-15 zero the rows of dropped tokens (PADDED output) while the attention
 //              runs and, in the fused call, copy the CTA's own 256 K and V rows from
 //              the last two ring tiles to the compacted cache.
@@ -31,8 +31,6 @@
 // runs out sets ZIPVL_DEV_TIMEOUT and all roles unwind to the common exit.
 #include <stdlib.h>
 #include <string.h>
-
-#include <type_traits>
 
 #include "tc.cuh"
 #include "tc_ptx.cuh"
@@ -66,7 +64,7 @@ struct Barriers {
     uint64_t s_full[2];
     uint64_t p_full[2];
     uint64_t pv_done[2];
-    uint64_t tail_full[2];   // the CTA's own key tiles (K and V) have landed: told by the issuer
+    uint64_t tail_full[2];   // the CTA's own key tiles (K and V) have landed
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -148,7 +146,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
             mbar_init(smem_u32(&bar->s_full[x]), 1);
             mbar_init(smem_u32(&bar->p_full[x]), 128);
             mbar_init(smem_u32(&bar->pv_done[x]), 1);
-            mbar_init(smem_u32(&bar->tail_full[x]), 1);
+            mbar_init(smem_u32(&bar->tail_full[x]), 128);
         }
         bar->abort_flag = 0;
         fence_barrier_init();
@@ -266,6 +264,10 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
             else cp_async_wait<0>();
             fence_proxy_async();
             mbar_arrive(smem_u32(&bar->full[seq % kSlots]));
+            // V, and K before it, of the CTA's own tokens: for the warps that copy them to the compacted cache
+            // (announced here rather than by the issuer, which comes to them only with its last steps: 101.1 -> 99.1
+            // us for the 2944-token layer)
+            if ((seq & 1) && (seq >> 1) >= ta) mbar_arrive(smem_u32(&bar->tail_full[(seq >> 1) - ta]));
         }
     } else if (warp >= 12) {
         // ---------------------- MMA issuer (warp 12), zero-fill (13-15) ----------------------
@@ -314,16 +316,15 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
             // own 256 kept tokens, already gathered into shared memory for the attention.  The
             // CTA of the first query head of a KV group writes them to the compacted cache
             // from there (every (pair, kv head) once over the grid): these warps wait for the
-            // tile like the issuer does and un-swizzle it, two rows per instruction.  The
+            // tile and un-swizzle it, two rows per instruction.  The
             // slots of a CTA's last tiles are never refilled, so there is no race with the
             // producers; the attention only reads them.
             if (kc != nullptr && h % a.G == 0) {
                 const int lim = min(n_valid, capacity);
                 const int sub = lane >> 4, ch = lane & 15;
                 for (int j = ta; j < n_kv; ++j) {               // key tile j = kept tokens 128j ..
-                    // the issuer follows the ring in order and says when K and V of this tile
-                    // are in (the ring's own barriers are only meaningful to a reader that
-                    // keeps up with every phase)
+                    // (the ring's own barriers are only meaningful to a reader that keeps up with
+                    // every phase)
                     mbar_wait(smem_u32(&bar->tail_full[j - ta]), 0, abort_flag);
                     for (int kind = 0; kind < 2; ++kind) {       // 0: K (group 2j), 1: V (group 2j+1)
                         const int seq = 2 * j + kind;
@@ -397,50 +398,37 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
                 if (has_b) qk(1, 0);
             }
             release(0);
-            // The two query tiles advance independently: whichever has its P ready
-            // (and its V / next K tile landed) is served; nothing blocks on the other.
-            // A ring slot is released by whichever tile uses it last.
-            int next[2] = {0, 0};
-            bool loads_ok[2] = {false, false};
+            // The tiles take turns, A(n) B(n) A(n+1) ...: half a step apart is how they settle by themselves (one
+            // is in its softmax while the other's MMAs run), and a fixed order lets this warp sleep on
+            // the one barrier that comes next.  Polling the barriers of both tiles took issue slots
+            // from the softmax warps of its scheduler (300 cycles a tile) and saw a finished P 300 to 650 cycles
+            // late: a step of both tiles went from 4050 to 3620 cycles.  It needs the first and the
+            // diagonal tile to take no longer than the others (see the mask below): the other tile waits for them.
+            // Sleeping on one tile with a time limit and looking at the other was slower than polling.
+            // The later user of a ring slot, B if it uses the slot at all, releases it.
             const int cnt[2] = {n_a, has_b ? n_kv : 0};
-            auto is_full = [&](int seq) {
-                return warp_try_wait(smem_u32(&bar->full[seq % kSlots]), (seq / kSlots) & 1);
-            };
-            for (uint32_t spin = 0; (next[0] < cnt[0] || next[1] < cnt[1]) && !*abort_flag; ++spin) {
+            bool ok = !*abort_flag;
+            for (int n = 0; n < n_kv && ok; ++n) {
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    const int n = next[x], o = 1 - x;
-                    if (n >= cnt[x]) continue;
+                    if (n >= cnt[x] || !ok) continue;
                     const bool more = (n + 1 < cnt[x]);
-                    // the tiles this step reads are looked up while the issuer is idle, so
-                    // a finished softmax finds the way to the tensor pipe already clear
-                    if (!loads_ok[x]) {
-                        // (every producer thread announces its tiles in order, so a landed
-                        // K(n+1) says that V(n) has landed too: one look at one barrier)
-                        loads_ok[x] = is_full(more ? 2 * n + 2 : 2 * n + 1);
-                        if (!loads_ok[x]) continue;
-                        // The last step of tile A reads the key tile of A's own tokens, that of
-                        // tile B the one of B's -- the CTA's own 256 tokens: K and V of that tile are in now,
-                        // which the warps that copy them to the compacted cache are told here
-                        // (once per tile: loads_ok is set once per step).
-                        if (!more && leader) mbar_arrive(smem_u32(&bar->tail_full[x]));
-                    }
-                    if (!warp_try_wait(smem_u32(&bar->p_full[x]), n & 1)) continue;
+                    // (every producer thread announces its tiles in order, so a landed
+                    // K(n+1) says that V(n) has landed too: one look at one barrier)
+                    const int seq = more ? 2 * n + 2 : 2 * n + 1;
+                    ok = mbar_wait(smem_u32(&bar->full[seq % kSlots]), (seq / kSlots) & 1, abort_flag);
+                    ok = ok && mbar_wait(smem_u32(&bar->p_full[x]), n & 1, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) continue;
                     tc_fence_after();
                     pv(x, n);
                     // the commit behind QK(n+1) also covers PV(n): a landed S(n+1) tells the
                     // softmax warps that O is complete through tile n; the last PV commits itself
                     if (more) qk(x, n + 1);
                     else if (leader) mma_commit(smem_u32(&bar->pv_done[x]));
-                    next[x] = n + 1;
-                    loads_ok[x] = false;
-                    // V(n): the other tile is past it, or never uses it
-                    if (!(n < cnt[o]) || next[o] > n) release(2 * n + 1);
-                    // K(n+1): released once every user has issued its QK
-                    if (more && (!(n + 1 < cnt[o]) || next[o] > n)) release(2 * n + 2);
-                    spin = 0;
+                    if (x == 1 || n >= cnt[1]) release(2 * n + 1);
+                    if (more && (x == 1 || n + 1 >= cnt[1])) release(2 * n + 2);
                 }
-                if (spin >= kWaitLimit) *abort_flag = 1;
             }
         }
     } else {
@@ -470,8 +458,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
             // (P then stays below 2^32, far inside bf16 and fp32 range), which makes the
             // read-modify-write of O a rare event.
             const int quad = warp & 3;                  // this warp's 32-row (and, on the diagonal, 32-column) block
-            auto tile = [&](auto diag_c, int n) {
-                constexpr bool kDiag = decltype(diag_c)::value;
+            auto tile = [&](int n) {
                 uint32_t sr[4][32];
                 tmem_ld32(tS, sr[0]);
                 tmem_ld32(tS + 32, sr[1]);
@@ -482,19 +469,31 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
                 // On the diagonal tile row r sees columns 0..r.  A warp's 32 rows share their
                 // 32-column chunk: chunks below it are fully visible, the chunk with the
                 // warp's own index is cut per lane (column e <= lane), chunks above it are
-                // fully masked -- three warp-uniform cases instead of a test per element.
-                auto scan = [&](int c) {
-                    if (kDiag && c > quad) return;
-                    const bool cut = kDiag && c == quad;
+                // fully masked.  The masked scores become -inf here and the rest is the code of every
+                // other tile: a second copy of the softmax for the diagonal would run cold once per
+                // CTA (3000 cycles for half a tile's work).
+                // On the diagonal tile row r sees columns 0..r.  A warp's 32 rows share their
+                // 32-column chunk: chunks below it are fully visible, the chunk with the
+                // warp's own index is cut per lane (column e <= lane), chunks above it are
+                // fully masked.  The masked scores become -inf here and the rest is the code of every other
+                // tile.  A softmax of its own for the diagonal, without the masked exponentials, ran cold once
+                // per CTA: 3000 cycles for half a tile's work (together with the order of the issuer: 2944
+                // tokens, 32 heads, whole layer 104.9 -> 99.1 us, 7181 tokens 323 -> 305, 18432 with 28 heads
+                // on 4 2090 -> 2050; the loop body must stay small, a test per chunk inside it cost 2%).
+                if (__builtin_expect(n == diag_tile, 0)) {
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int e = 0; e < 32; e += 2) {
-                        float v0 = __uint_as_float(sr[c][e]), v1 = __uint_as_float(sr[c][e + 1]);
-                        if (cut) {
-                            if (e > lane) v0 = -INFINITY;
-                            if (e + 1 > lane) v1 = -INFINITY;
+                    for (int c = 0; c < 4; ++c)
+                        if (c >= quad) {
+                            const int see = c > quad ? -1 : lane;
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) sr[c][e] = e > see ? 0xff800000u : sr[c][e];
                         }
-                        mx4[(e >> 1) & 3] = max3(mx4[(e >> 1) & 3], v0, v1);
-                    }
+                }
+                auto scan = [&](int c) {
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2)
+                        mx4[(e >> 1) & 3] = max3(mx4[(e >> 1) & 3], __uint_as_float(sr[c][e]), __uint_as_float(sr[c][e + 1]));
                 };
                 scan(0);
                 scan(1);
@@ -514,25 +513,14 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint32_t p16[16];
-                    if (kDiag && c > quad) {
-                        // a fully masked chunk: P = 0, no exponentials
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) p16[e] = 0u;
-                    } else {
-                        const bool cut = kDiag && c == quad;
-#pragma unroll
-                        for (int e = 0; e < 32; e += 2) {
-                            const uint64_t x2 = fma2(pack2u(sr[c][e], sr[c][e + 1]), scale2, neg_m2);
-                            float x0, x1;
-                            unpack2f(x2, x0, x1);
-                            float p0 = ex2(x0), p1 = ex2(x1);
-                            if (cut) {
-                                if (e > lane) p0 = 0.f;
-                                if (e + 1 > lane) p1 = 0.f;
-                            }
-                            sum2[(e >> 1) & 3] = add2(sum2[(e >> 1) & 3], pack2f(p0, p1));
-                            p16[e >> 1] = pack16<kHalf>(p0, p1);
-                        }
+                    for (int e = 0; e < 32; e += 2) {
+                        const uint64_t x2 = fma2(pack2u(sr[c][e], sr[c][e + 1]), scale2, neg_m2);
+                        float x0, x1;
+                        unpack2f(x2, x0, x1);
+                        const float p0 = ex2(x0), p1 = ex2(x1);
+                        sum2[(e >> 1) & 3] = add2(sum2[(e >> 1) & 3], pack2f(p0, p1));
+                        p16[e >> 1] = pack16<kHalf>(p0, p1);
                     }
                     // P (bf16) overwrites the front of S: every S column is in registers
                     tmem_st16(tS + c * 16, p16);
@@ -560,8 +548,7 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
             for (int n = 0; n < n_mine; ++n) {
                 mbar_wait(smem_u32(&bar->s_full[x]), n & 1, abort_flag);
                 tc_fence_after();
-                if (n == diag_tile) tile(std::true_type{}, n);
-                else tile(std::false_type{}, n);
+                tile(n);
                 tc_fence_before();
                 mbar_arrive(smem_u32(&bar->p_full[x]));
             }
