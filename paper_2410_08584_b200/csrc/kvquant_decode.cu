@@ -5,22 +5,27 @@
 // What bounds it: a cached value is 2 or 4 bits, so one SM has to get through about 45 values per
 // cycle to keep up with HBM.  With a shift, a conversion and a multiply-add per value and query
 // head on the CUDA cores the step took 75 us for six requests of 1.4K-5.9K tokens, 32 heads
-// (1.1 TB/s); this kernel and the merge behind it take 30 us, and 126 us (4.9 TB/s of codes and parameters)
-// for 23 requests of 5.6K-7.6K tokens.  Here the contractions run on the tensor cores straight from registers (mma.sync
-// m16n8k16: the operand is unpacked in registers and used once, a tcgen05 operand would have to go
-// through shared memory first), and unpacking costs one AND per two values:
-//   - a code c at bit p of a 16-bit half is the IEEE half number c * 2^(p-24) -- a subnormal, which
-//     the tensor core takes exactly -- for every p up to 8; the factor 2^p is taken out of the other
-//     operand (q) or of the result (o);
+// (1.1 TB/s); this kernel and the merge behind it take 36.6 us.  Here the contractions run on the tensor cores
+// straight from registers (mma.sync m16n8k16: the operand is unpacked in registers and used once, a tcgen05 operand
+// would have to go through shared memory first), and unpacking costs three instructions per four values:
+//   - a code c at bit p of a 16-bit half, with the exponent of 2^(10 - p) put above it, is the IEEE half number
+//     2^(10 - p) + c; a packed subtraction leaves c - centre, exactly (centre: 8 of 0..15, 2 of 0..3).
+//     Left as a subnormal, c * 2^(p - 24), a code needs no subtraction, but the tensor core lines products
+//     up by their nominal exponents and cuts off below: such codes lose up to ten bits of the sum (30 us per step instead
+//     of 36.6, errors of the fp32 results 10 to 130 times those of a plain fp32 evaluation);
 //   - the order of the 16 contraction indices of an MMA is free as long as both operands share it, so a
 //     lane takes whole 32-bit words of a row and the halves of a word pair up by themselves;
 //   - S = Q K^T: A = codes [16 rows x 16 channels], B = q [16 channels x 8 columns = query heads], q in
 //     half precision scaled by a power of two per head (exact for bfloat16 and half values down to
-//     2^-18 of the largest; fp32 accumulation);
+//     2^-28 of the largest; fp32 accumulation);
 //   - O = P V: A = codes [16 channels x 16 rows], B = p * v_scale [16 rows x 8 columns], split into
-//     two half numbers, w = hi + lo, in columns g and g + 4: 22 bits of the weight, absolute error 2^-33 of
-//     the largest one;
-//   - k^ = code * s + z adds z * sum(q) to a score and p * z to every channel of the output.
+//     two half numbers, w = hi + 2^-11 lo, in columns g and g + 4: 22 bits of a weight down to 2^-22 of
+//     the largest, 2^-44 of that below.  The products are exact; p is the one that the denominator adds up;
+//   - k^ = (code - centre) * s + (z + centre * s): the second term adds sum(q) times itself to a score and p times itself
+//     to every channel of the output.  With the codes centred both sums stay near the results and nothing
+//     large has to cancel: the tensor core cuts its sums off instead of rounding them, 2^-23 of the running
+//     sum per MMA.  Error of the fp32 results against 64 bits, N(0, 1) keys and values, queries of four sizes,
+//     1.4K to 9K rows: 0.2 to 0.9 of that of the plain fp32 evaluation that this kernel replaced.
 // A warp owns a chunk of rows of one (request, kv head); the four warps of a CTA take four
 // neighbouring heads of the same rows (their parameters share 32-byte sectors).  32 rows per step: each
 // lane evaluates the softmax weight of one row (the query repeated over the columns brings a
@@ -38,12 +43,19 @@ namespace kvq {
 namespace {
 
 constexpr int kWarps = 4, kStages = 3;
+constexpr float kLowScale = 2048.f;          // of the low part of a weight, which would be subnormal otherwise
 template <int D> struct Ring { static constexpr int kBytes = kStages * (2 * 32 * (D / 2) + 256); };   // per warp, 4-bit rows
 
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the same with a sum of its own, d = a b + c
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1, float c0, float c1, float c2, float c3) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
 }
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
     const __half2 h = __floats2half2_rn(lo, hi);
@@ -56,17 +68,24 @@ __device__ __forceinline__ float pow2(int e) {
 }
 
 // The i-th code pair of a 32-bit word of 16-bit halves with BITS-bit codes: codes i and i + 16 / BITS
-// of the word (one from each half) as two half numbers c * 2^(shift_of(i) - 24).  Bits 0..9 of a half are its
-// mantissa, so codes at bit 8 (2 bits wide) or 4 (4 bits wide) still read linearly; the ones above
-// are moved down first.
+// of the word (one from each half), less kCentre, as two half numbers.  A code c at bit p of a half's mantissa,
+// with the exponent bits of 2^(10 - p) put above it, reads 2^(10 - p) + c; taking 2^(10 - p) + kCentre off is exact.
+// Bits 0..9 are the mantissa; the codes above it are moved down first.
 template <int BITS>
-__device__ __forceinline__ constexpr int pair_shift(int i) { return BITS == 4 ? 4 * (i & 1) : (i < 5 ? 2 * i : 2 * (i - 5)); }
-template <int BITS>
-__device__ __forceinline__ uint32_t code_pair(uint32_t w, int i) {
-    const uint32_t moved = (BITS == 4) ? (i >= 2 ? w >> 8 : w) : (i >= 5 ? w >> 10 : w);
-    const uint32_t one = BITS == 4 ? 0x000f000fu : 0x00030003u;
-    return moved & (one << pair_shift<BITS>(i));
-}
+struct Code {
+    static constexpr int kCentre = 1 << (BITS - 1);
+    static __device__ __forceinline__ uint32_t pair(uint32_t w, int i) {
+        const int p = BITS == 4 ? 4 * (i & 1) : (i < 5 ? 2 * i : 2 * (i - 5));
+        const uint32_t moved = (BITS == 4) ? (i >= 2 ? w >> 8 : w) : (i >= 5 ? w >> 10 : w);
+        const uint32_t both = 0x00010001u;
+        const uint32_t raised = (moved & ((BITS == 4 ? 15u : 3u) * both << p)) | (uint32_t)(25 - p) * (both << 10);
+        // 2^(10 - p) + kCentre: its mantissa is kCentre at bit p
+        const uint32_t off = ((uint32_t)(25 - p) * (both << 10)) | ((uint32_t)kCentre * both << p);
+        uint32_t d;
+        asm("sub.f16x2 %0, %1, %2;" : "=r"(d) : "r"(raised), "r"(off));
+        return d;
+    }
+};
 
 // W consecutive 32-bit words (or one 16-bit half, W == 0) of shared memory
 template <int W>
@@ -142,6 +161,7 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
     constexpr int RB = D * BITS / 8;         // bytes of a row
     constexpr int PER = 16 / BITS;           // codes per 16-bit half
     constexpr int KS = D / 16;
+    constexpr float kCentre = Code<BITS>::kCentre;
     if (r0 >= r1) return;
     const int g = lane >> 2, t = lane & 3;
     // ---- the warp's ring of kStages steps: 32 rows of K, of V and their parameters each, fetched 16
@@ -181,7 +201,7 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
     for (int i = 0; i < kStages - 1; ++i) fetch(i);
     // ---- the query as B operand: head g & (G-1)'s channels D/4 * t ..., paired like the codes of K's words
     uint32_t qf[KS][2];
-    float k_factor[NH], q_sum[NH];           // dot * k_factor = scale_log2 * <q, code>; scale_log2 * sum(q)
+    float k_factor[NH], q_sum[NH];           // dot * k_factor = scale_log2 * <q, code - centre>; scale_log2 * sum(q)
     {
         float mx = 0.f, sum = 0.f;
         float x[D / 4];
@@ -211,10 +231,9 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
                     const int i = 2 * s + b, c = j * 2 * PER + i;
-                    const float d = f * (1.f / (float)(1 << pair_shift<BITS>(i)));
-                    qf[j * (PER / 2) + s][b] = pack_half2(x[c] * d, x[c + PER] * d);
+                    qf[j * (PER / 2) + s][b] = pack_half2(x[c] * f, x[c + PER] * f);
                 }
-        const float kf = pow2(24 - up) * scale_log2, qs = sum * scale_log2;
+        const float kf = pow2(-up) * scale_log2, qs = sum * scale_log2;
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
             const int src = 4 * (h + (G == 4 ? 2 * (t & 1) : 0));
@@ -247,38 +266,39 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
         uint32_t kw[2][2][KW];
 #pragma unroll
         for (int u = 0; u < 4; ++u) load_words<KW>(buf + (g + 8 * u) * RB + t * (KW * 4), kw[u >> 1][u & 1]);
-        // ---- scores of 2 x 16 rows
+        // ---- scores of 2 x 16 rows, two chains of MMAs side by side
         float c[2][4];
 #pragma unroll
-        for (int tile = 0; tile < 2; ++tile) {
+        for (int j = 0; j < KW; ++j)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) c[tile][e] = 0.f;
+            for (int s = 0; s < PER / 2; ++s) {
+                const int i = j * (PER / 2) + s;
 #pragma unroll
-            for (int j = 0; j < KW; ++j)
-#pragma unroll
-                for (int s = 0; s < PER / 2; ++s) {
+                for (int tile = 0; tile < 2; ++tile) {
                     const uint32_t w0 = kw[tile][0][j], w1 = kw[tile][1][j];
-                    const uint32_t a[4] = {code_pair<BITS>(w0, 2 * s), code_pair<BITS>(w1, 2 * s),
-                                           code_pair<BITS>(w0, 2 * s + 1), code_pair<BITS>(w1, 2 * s + 1)};
-                    mma16816(c[tile], a, qf[j * (PER / 2) + s][0], qf[j * (PER / 2) + s][1]);
+                    const uint32_t a[4] = {Code<BITS>::pair(w0, 2 * s), Code<BITS>::pair(w1, 2 * s),
+                                           Code<BITS>::pair(w0, 2 * s + 1), Code<BITS>::pair(w1, 2 * s + 1)};
+                    if (i == 0) mma16816(c[tile], a, qf[i][0], qf[i][1], 0.f, 0.f, 0.f, 0.f);
+                    else mma16816(c[tile], a, qf[i][0], qf[i][1]);
                 }
-        }
+            }
         uint2 pr[NT];
 #pragma unroll
         for (int u = 0; u < NT; ++u) pr[u] = *reinterpret_cast<const uint2 *>(buf + 64 * RB + item_row(u) * 8);
         // ---- this lane's weights
-        float sc[NT][NH], ev[NT], fv[NT];
+        float sc[NT][NH], ev[NT], fv[NT], vc[NT];
         bool grow = false;
 #pragma unroll
         for (int u = 0; u < NT; ++u) {
             const float ks = storage_to_float<kHalf>((unsigned short)(pr[u].x & 0xffffu));
-            const float kz = storage_to_float<kHalf>((unsigned short)(pr[u].x >> 16));
+            const float kz = fmaf(kCentre, ks, storage_to_float<kHalf>((unsigned short)(pr[u].x >> 16)));
             const float vs = storage_to_float<kHalf>((unsigned short)(pr[u].y & 0xffffu));
             // v scale = fv * 2^ev, fv in [1, 2) (a zero or subnormal scale: ev = -126)
             const uint32_t e = __float_as_uint(vs) >> 23;
             ev[u] = (float)(int)max(e, 1u) - 127.f;
             fv[u] = e - 1u < 254u ? __uint_as_float((__float_as_uint(vs) & 0x7fffffu) | 0x3f800000u)
                                   : (e == 0u ? vs * 8.507059e37f : vs);
+            vc[u] = fmaf(kCentre, vs, storage_to_float<kHalf>((unsigned short)(pr[u].y >> 16)));
             const bool in = base + item_row(u) < r1;
 #pragma unroll
             for (int h = 0; h < NH; ++h) {
@@ -320,10 +340,14 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
             for (int u = 0; u < NT; ++u) {
                 const float p = fast_exp2(sc[u][h] - ref);
                 st.l[h] += p;
-                st.zacc[h] = fmaf(p, storage_to_float<kHalf>((unsigned short)(pr[u].y >> 16)), st.zacc[h]);
-                const float w = fast_exp2(sc[u][h] + ev[u] - ref_w) * fv[u];     // below 2^16
+                st.zacc[h] = fmaf(p, vc[u], st.zacc[h]);
+                // p * v scale as a multiple of 2^ref_w, below 2^15 (a power of two of its own, not an exponential of
+                // its own: numerator and denominator of the softmax share the rounding of p)
+                const float up = ev[u] + (ref - ref_w);
+                float w = p * fv[u] * fast_exp2(fminf(up, 126.f));
+                if (up > 126.f) w *= fast_exp2(fminf(up - 126.f, 126.f));
                 const float hi = __half2float(__float2half_rn(w));
-                packed[u][h] = pack_half2(w, w - hi);
+                packed[u][h] = pack_half2(w, (w - hi) * kLowScale);
             }
         }
 #pragma unroll
@@ -348,7 +372,7 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 load_words<VW>(buf + 32 * RB + (8 * tile + t + 4 * (u >> 1) + 16 * (u & 1)) * RB + g * (VW ? VW * 4 : 2), vw[u]);
-            // ---- O += codes^T w: per MMA two channels of this lane's channel group, 16 rows
+            // ---- O += (codes - kCentre)^T w: per MMA two channels of this lane's channel group, 16 rows
             // (pairs of rows 2t, 2t + 1 and 2t + 8, 2t + 9 share a word after a byte permutation)
 #pragma unroll
             for (int j = 0; j < VN; ++j)
@@ -358,8 +382,8 @@ __device__ __forceinline__ void run_block(Warp<D, G> &st, const unsigned char *k
                     const uint32_t x1 = __byte_perm(vw[2][j], vw[3][j], half ? 0x7632 : 0x5410);
 #pragma unroll
                     for (int s = 0; s < PER / 2; ++s) {
-                        const uint32_t a[4] = {code_pair<BITS>(x0, 2 * s), code_pair<BITS>(x0, 2 * s + 1),
-                                               code_pair<BITS>(x1, 2 * s), code_pair<BITS>(x1, 2 * s + 1)};
+                        const uint32_t a[4] = {Code<BITS>::pair(x0, 2 * s), Code<BITS>::pair(x0, 2 * s + 1),
+                                               Code<BITS>::pair(x1, 2 * s), Code<BITS>::pair(x1, 2 * s + 1)};
                         mma16816(st.o[(j * 2 + half) * (PER / 2) + s], a, b[0], b[1]);
                     }
                 }
@@ -433,12 +457,6 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
     for (int h = 0; h < NH; ++h) { st.m[h] = -INFINITY; st.m_w[h] = -INFINITY; st.l[h] = 0.f; st.zacc[h] = 0.f; }
     run_block<4, kHalf, D, G>(st, qb.k_hi, qb.v_hi, qb.p_hi, c0, min(c1, n_hi), Hkv, hkv, qh, scale_log2, ring, lane,
                               mine ? &fresh : nullptr);
-    // the accumulators carry 2^(bit position - 24) of their block's codes
-#pragma unroll
-    for (int s = 0; s < VS; ++s)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            st.o[s][e] *= (float)(1 << pair_shift<2>((2 * s + (e >> 1)) % 8)) / (float)(1 << pair_shift<4>((2 * s + (e >> 1)) % 4));
     run_block<2, kHalf, D, G>(st, qb.k_lo, qb.v_lo, qb.p_lo, max(c0 - n_hi, 0), c1 - n_hi, Hkv, hkv, qh, scale_log2, ring, lane);
 
     // ---- this chunk's (m, l, o): o = sum p * (code * v_scale + v_zero).  Lane t < 2 holds the hi parts of
@@ -447,17 +465,16 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
 #pragma unroll
     for (int h = 0; h < NH; ++h) {
         const float l = reduce<G>(st.l[h], add), z = reduce<G>(st.zacc[h], add);
-        // from the accumulators' reference (and 2^8) to p's; 2^24 from the codes' bit position
-        const float up = fast_exp2(st.m_w[h] - st.m[h] + 16.f);
+        // from the accumulators' reference (and 2^8) to p's
+        const float up = fast_exp2(st.m_w[h] - st.m[h] - 8.f);
         const bool write = t < 2 && 2 * t + h < G;
         float *row = dst + (2 * t + h) * head_pitch;
         if (write && g == 0) *reinterpret_cast<float2 *>(row) = make_float2(st.m[h], l);
 #pragma unroll
         for (int s = 0; s < VS; ++s) {
-            const float a = st.o[s][h] + __shfl_xor_sync(0xffffffffu, st.o[s][h], 2);
-            const float c = st.o[s][2 + h] + __shfl_xor_sync(0xffffffffu, st.o[s][2 + h], 2);
-            const float fa = 1.f / (float)(1 << pair_shift<2>((2 * s) % 8)), fc = 1.f / (float)(1 << pair_shift<2>((2 * s + 1) % 8));
-            if (write) *reinterpret_cast<float2 *>(row + 2 + g * (D / 8) + 2 * s) = make_float2(fmaf(a * fa, up, z), fmaf(c * fc, up, z));
+            const float a = fmaf(__shfl_xor_sync(0xffffffffu, st.o[s][h], 2), 1.f / kLowScale, st.o[s][h]);
+            const float c = fmaf(__shfl_xor_sync(0xffffffffu, st.o[s][2 + h], 2), 1.f / kLowScale, st.o[s][2 + h]);
+            if (write) *reinterpret_cast<float2 *>(row + 2 + g * (D / 8) + 2 * s) = make_float2(fmaf(a, up, z), fmaf(c, up, z));
         }
     }
 }
