@@ -10,6 +10,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from parity import to_np
 
 pytestmark = pytest.mark.gpu
@@ -76,3 +77,44 @@ def test_quantised_scores_that_agree(zipvl, dtype, d, bits):
     bound = np.log(2) * (d / 16) * 2.0 ** -24 * partial
     err = np.abs(out.astype(np.float64)).max(-1)
     assert np.sqrt(np.mean(err ** 2)) < np.sqrt(np.mean(bound ** 2))
+
+
+def plain_step(z, q, k, v, dtype):
+    """q [B, H, d] over caches k, v [B, L, H, d]; also the exact result."""
+    B, L, H, d = k.shape
+    off = torch.arange(B) * L * H * d
+    n = torch.full((B,), L, dtype=torch.int32)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    desc = z.zipvl_decode_desc(B, H, H, d, CODE[dtype], 0.0)
+    out = z.zipvl_decode(desc, q.to(DEV), None, None, k.to(DEV), v.to(DEV), off.to(DEV), n.to(DEV), n.to(DEV), L, status=st)
+    assert st.item() == 0
+    want = oracle.decode_step(to_np(q), None, None, to_np(k).ravel().copy(), to_np(v).ravel().copy(), off.numpy(), n.numpy().copy(), H)
+    return to_np(out), want
+
+
+@pytest.mark.parametrize("dtype,bits", [(torch.bfloat16, 8), (torch.float16, 11)])
+@pytest.mark.parametrize("d", [64, 96, 128])
+def test_small_weights_count(zipvl, dtype, bits, d):
+    """Every sixteenth row has 2^26 times the weight of the others and a value of zero: the output is what the small
+    weights add up to.  Bound: the output's rounding, and four units of the last of 24 bits."""
+    L, H = 700, 3
+    q = torch.ones(1, H, d, dtype=dtype)
+    k = torch.zeros(1, L, H, d, dtype=dtype)
+    v = torch.full((1, L, H, d), 30000.0).to(dtype)
+    k[:, ::16] = 26 * np.log(2) / np.sqrt(d)
+    v[:, ::16] = 0
+    out, want = plain_step(zipvl, q, k, v, dtype)
+    assert np.abs(out / want - 1).max() < 2.0 ** -bits + 4 * 2.0 ** -24 * 26
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+def test_sums_that_grow_and_cancel(zipvl, dtype):
+    """The second half of a cache repeats the first with the values negated: sums over a warp's rows grow to half a value's
+    size and go back to zero.  Rounded sums over its sixteen tiles are off by 2^-25 of that each, at random."""
+    B, L, H, d = 16, 1024, 32, 128
+    g = torch.Generator().manual_seed(5)
+    k = torch.randn(B, L // 2, H, d, generator=g).repeat(1, 2, 1, 1).to(dtype)
+    v = (1 + 0.1 * torch.randn(B, L // 2, H, d, generator=g)).to(dtype)
+    q = (0.1 * torch.randn(B, H, d, generator=g)).to(dtype)
+    out, _ = plain_step(zipvl, q, k, torch.cat([v, -v], 1), dtype)
+    assert np.sqrt(np.mean(out.astype(np.float64) ** 2)) < np.sqrt(16) * 2.0 ** -25 * 0.5
