@@ -77,7 +77,10 @@ __device__ __forceinline__ uint32_t transpose8(uint32_t x) {
 // x to its leading eight bits, as the storage type holds them (a subnormal half holds fewer)
 template <bool kHalf>
 __device__ __forceinline__ float leading_bits(float x) {
-    if (kHalf) return __half2float(__float2half_rn(__uint_as_float(__float_as_uint(x) & 0xffff0000u)));
+    if (kHalf) {     // (2^-24 at least, of a positive number: a weight may meet an infinite value)
+        const float y = __half2float(__float2half_rn(__uint_as_float(__float_as_uint(x) & 0xffff0000u)));
+        return x > 0.f ? fmaxf(y, 5.9604645e-8f) : y;
+    }
     return __bfloat162float(__float2bfloat16_rn(x));
 }
 template <int W>
@@ -218,7 +221,12 @@ decode_mma_kernel(DmArgs a) {
             const int r = min(2 * t + (u & 1) + 8 * (u >> 1), c1 - 1 - base);
             const char *p = (base + r == new_row ? vn : vb + off + r * pitch) + g * (VW * 4);
 #pragma unroll
-            for (int j = 0; j < VJ; ++j) load_row(p + j * (VW * 32), vr[u][j]);
+            for (int j = 0; j < VJ; ++j) {
+                if (2 * t + (u & 1) + 8 * (u >> 1) < c1 - base) load_row(p + j * (VW * 32), vr[u][j]);
+                else
+#pragma unroll
+                    for (int w = 0; w < VW; ++w) vr[u][j][w] = 0u;
+            }
         }
     };
     int base = c0 + warp * 16;
@@ -341,7 +349,13 @@ decode_mma_kernel(DmArgs a) {
     }
 
     // ---- merge the warps, eight heads at a time (one head: the parts of its weights first)
+    const auto channel = [&](int s) { return (s / VW) * (16 * VW) + g * (2 * VW) + (s % VW) * 2; };
     if (kOne) {
+        // what the first parts alone make goes into a free place: an infinite value is infinite there, where the
+        // parts that are zero or negative make it NaN
+        if (t == 0)
+#pragma unroll
+            for (int s = 0; s < VS; ++s) *reinterpret_cast<float2 *>(&sm_o[warp][1][channel(s)]) = make_float2(o[0][s][0], o[0][s][2]);
 #pragma unroll
         for (int s = 0; s < VS; ++s)
 #pragma unroll
@@ -361,8 +375,7 @@ decode_mma_kernel(DmArgs a) {
             if (g == 0) { sm_m[warp][2 * t + h] = m[nt][h]; sm_l[warp][2 * t + h] = l[nt][h]; }
 #pragma unroll
             for (int s = 0; s < VS; ++s) {
-                const int ch = (s / VW) * (16 * VW) + g * (2 * VW) + (s % VW) * 2;
-                *reinterpret_cast<float2 *>(&sm_o[warp][2 * t + h][ch]) = make_float2(o[nt][s][h], o[nt][s][2 + h]);
+                *reinterpret_cast<float2 *>(&sm_o[warp][2 * t + h][channel(s)]) = make_float2(o[nt][s][h], o[nt][s][2 + h]);
             }
         }
         __syncthreads();
@@ -379,6 +392,16 @@ decode_mma_kernel(DmArgs a) {
                 L = fmaf(f, sm_l[w][h], L);
                 x = fmaf(f, v.x, x);
                 y = fmaf(f, v.y, y);
+            }
+            if (kOne && !(fabsf(x) + fabsf(y) < INFINITY)) {
+                float u = 0.f, v = 0.f;
+                for (int w = 0; w < kWarps; ++w) {
+                    const float f = sm_m[w][h] == -INFINITY ? 0.f : fast_exp2(sm_m[w][h] - M);
+                    u = fmaf(f, sm_o[w][1][ch], u);
+                    v = fmaf(f, sm_o[w][1][ch + 1], v);
+                }
+                if (!(fabsf(u) < INFINITY)) x = u;
+                if (!(fabsf(v) < INFINITY)) y = v;
             }
             float *p = dst + (nt * 8 + h) * head_pitch;
             *reinterpret_cast<float2 *>(p + 2 + ch) = make_float2(x, y);
