@@ -228,8 +228,11 @@ prefill_simt_kernel(LayerArgs a, const T *__restrict__ q, const T *__restrict__ 
         }
         if (more) ptx::cp_async_wait<1>(); else ptx::cp_async_wait<0>();   // V is in
         __syncthreads();
+        // Keys behind the warp's last row weigh nothing and are left out: 0 x Inf would reach rows that do not see
+        // that key (rows of a warp are 4 RG consecutive ones, a multiple of four).
+        const int seen = min(kBN, i0 + ((tid >> 5) + 1) * (4 * RG) - kt * kBN);
 #pragma unroll 2
-        for (int j = 0; j < kBN; j += 4) {
+        for (int j = 0; j < seen; j += 4) {
             float4 p[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) p[i] = *reinterpret_cast<const float4 *>(Ps + (row0 + RG * i) * PP + j);

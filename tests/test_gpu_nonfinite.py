@@ -32,3 +32,21 @@ def test_infinite_value_in_a_cache(zipvl, dtype, H, Hkv, d, L, row):
     got, want = run(v), run(clean)
     want[:, 5], want[:H // Hkv, 7] = np.inf, -np.inf
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("d", [64, 96, 128])
+@pytest.mark.parametrize("n,row", [(40, 32), (150, 96), (64, 48), (200, 176), (1000, 720)])
+def test_infinite_value_in_a_prompt_fp32(zipvl, d, n, row):
+    """Rows in front of the token do not see its value: their outputs are the bits they are without it.  (Rows that
+    share its group of sixteen may meet it with weight zero; row is the first of one.)"""
+    z, H = zipvl, 2
+    g = torch.Generator().manual_seed(n + d)
+    q, k, v = (torch.randn(n, H, d, generator=g).to(DEV) for _ in range(3))
+    idx, count = torch.arange(n, dtype=torch.int32, device=DEV), torch.tensor([n], dtype=torch.int32, device=DEV)
+    lay = z.layer_desc(q, k)
+    want = z.zipvl_sparse_prefill(lay, q, k, v, idx, count, n).cpu()
+    bad = v.clone()
+    bad[row, :, 3] = float("inf")
+    got = z.zipvl_sparse_prefill(lay, q, k, bad, idx, count, n).cpu()
+    want[row:, :, 3] = float("inf")
+    assert torch.equal(got, want)
