@@ -296,9 +296,11 @@ zipvl_status zipvl_layer_step_host(const zipvl_layer *layer, const void *q, cons
         ZIPVL_CUDA(cudaStreamWaitEvent(c.out, c.chosen, 0));
         ZIPVL_CUDA(cudaMemcpyAsync(c.misc, d_misc, 16, cudaMemcpyDeviceToHost, c.out));
         ZIPVL_CUDA(cudaEventRecord(c.told, c.out));
-        // ---- in: V, then Q by groups of heads (rows already fetched are written again, with the same bytes)
+        // ---- in: V, then Q by groups of heads.  The copies write the probe rows of Q again, so they wait for the kernels
+        // that fetched and read them (which are done while V comes in, unless its heads are few)
         ZIPVL_CUDA(up(o_v, v, kb));
         ZIPVL_CUDA(cudaEventRecord(c.v_in, c.in));
+        if (m_q) ZIPVL_CUDA(cudaStreamWaitEvent(c.in, c.chosen, 0));
         if (m_q)
             for (int g = 0; g < groups; ++g) {
                 if (groups == 1) ZIPVL_CUDA(up(o_q, q, qb));
