@@ -11,6 +11,7 @@
 //     the full rate), the attention of a group runs as soon as it is there, and its output goes out while
 //     the next group comes in.
 // Three streams (in, run, out) joined by events; the host waits twice, for k and for the end.
+#include <cuda.h>
 #include <math.h>
 
 #include <mutex>
@@ -107,19 +108,31 @@ void give_context(int dev, HostContext &c) {
     c.destroy();
 }
 
-// The device's address of pinned host memory [p, p + bytes); nullptr for any other memory.
+// The device's address of pinned host memory [p, p + bytes); nullptr for any other memory.  The whole range has to
+// lie in one allocation: two pinned ranges may have memory between them that the GPU cannot read.
 const void *mapped(const void *p, size_t bytes) {
     if (!p) return nullptr;
-    cudaPointerAttributes first, last;
-    if (cudaPointerGetAttributes(&first, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, (const char *)p + bytes - 1) != cudaSuccess) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    const bool ok = first.type == cudaMemoryTypeHost && last.type == cudaMemoryTypeHost && first.devicePointer &&
-                    (const char *)last.devicePointer == (const char *)first.devicePointer + (bytes - 1) &&
-                    !((uintptr_t)first.devicePointer & 15u);
-    return ok ? first.devicePointer : nullptr;
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer || ((uintptr_t)at.devicePointer & 15u)) return nullptr;
+    static const auto attribute = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &f, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<CUresult (*)(void *, CUpointer_attribute, CUdeviceptr)>(f);
+    }();
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    const CUdeviceptr first = (CUdeviceptr)(uintptr_t)at.devicePointer;
+    if (!attribute || attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, first) != CUDA_SUCCESS ||
+        attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, first) != CUDA_SUCCESS)
+        return nullptr;
+    return first >= start && bytes <= size && first - start <= size - bytes ? at.devicePointer : nullptr;
 }
 
 // Small inputs read over the bus by the GPU itself.  Block r < P: probe row r of Q into its place; the blocks
