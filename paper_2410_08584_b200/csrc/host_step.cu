@@ -374,7 +374,11 @@ zipvl_status zipvl_layer_step_host(const zipvl_layer *layer, const void *q, cons
                                              cudaMemcpyDeviceToHost, c.out));
         }
         ZIPVL_CUDA(cudaMemcpyAsync(c.misc, d_misc, 16, cudaMemcpyDeviceToHost, c.out));
-        ZIPVL_CUDA(cudaStreamSynchronize(c.out));       // (everything on `in` and `run` is in front of it)
+        // (everything on `in` and `run` is in front of it; the free too is over when the call returns, so that
+        // zipvl_release_host_scratch finds the memory in the pool)
+        ZIPVL_CUDA(cudaFreeAsync(base, c.out));
+        base = nullptr;
+        ZIPVL_CUDA(cudaStreamSynchronize(c.out));
         if (k_out) *k_out = kept_rows;
         if (c.misc[2] != 0)
             return fail(c.misc[2] & ZIPVL_DEV_TIMEOUT ? ZIPVL_ERR_TIMEOUT : ZIPVL_ERR_BAD_INDEX,
@@ -382,9 +386,11 @@ zipvl_status zipvl_layer_step_host(const zipvl_layer *layer, const void *q, cons
         return ZIPVL_OK;
     };
     status = body();
-    if (status != ZIPVL_OK)                             // nothing may still be using the buffers
+    if (status != ZIPVL_OK) {                           // nothing may still be using the buffers
         for (cudaStream_t s : {c.in, c.run, c.out}) cudaStreamSynchronize(s);
-    if (base) cudaFreeAsync(base, c.out);
+        if (base) cudaFreeAsync(base, c.out);
+        cudaStreamSynchronize(c.out);
+    }
     give_context(dev, c);
     return status;
 }

@@ -99,3 +99,15 @@ def test_two_threads(zipvl):
         for turn in got[i]:
             for a, b in zip(turn, want[i]):
                 same(a, b)
+
+
+def test_scratch_is_given_back(zipvl):
+    """zipvl_release_host_scratch right behind a call leaves the device as much free memory as before the call."""
+    x = inputs(2945, 32, 32, 128, torch.bfloat16, 1)
+    from_the_host(zipvl, x, 0.9)
+    zipvl.zipvl_release_host_scratch()
+    before = torch.cuda.mem_get_info()[0]
+    for _ in range(5):
+        from_the_host(zipvl, x, 0.9)
+        zipvl.zipvl_release_host_scratch()
+        assert torch.cuda.mem_get_info()[0] >= before - (2 << 20)      # (the scratch is some 150 MB)
