@@ -15,7 +15,6 @@
 #include <math.h>
 
 #include <mutex>
-#include <vector>
 
 #include "common.cuh"
 #include "tc.cuh"
@@ -82,14 +81,18 @@ struct HostContext {
         for (int i = 0; i < kMaxGroups; ++i) { f(q_in[i]); f(done[i]); }
     }
 };
-std::vector<HostContext> g_host_context[kMaxDevices];
+// (a fixed array: nothing that may throw behind a C entry)
+struct KeptContexts {
+    HostContext at[kKeptContexts];
+    int n;
+} g_host_context[kMaxDevices];
 
 cudaError_t take_context(int dev, HostContext *c) {
     {
         std::lock_guard<std::mutex> lock(g_host_mutex);
-        if (!g_host_context[dev].empty()) {
-            *c = g_host_context[dev].back();
-            g_host_context[dev].pop_back();
+        KeptContexts &kept = g_host_context[dev];
+        if (kept.n > 0) {
+            *c = kept.at[--kept.n];
             return cudaSuccess;
         }
     }
@@ -100,8 +103,9 @@ cudaError_t take_context(int dev, HostContext *c) {
 void give_context(int dev, HostContext &c) {
     {
         std::lock_guard<std::mutex> lock(g_host_mutex);
-        if (g_host_context[dev].size() < kKeptContexts) {
-            g_host_context[dev].push_back(c);
+        KeptContexts &kept = g_host_context[dev];
+        if (kept.n < kKeptContexts) {
+            kept.at[kept.n++] = c;
             return;
         }
     }
@@ -178,8 +182,8 @@ zipvl_status zipvl_release_host_scratch(void) {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return fail(ZIPVL_ERR_CUDA, "zipvl_release_host_scratch: no current device");
     std::lock_guard<std::mutex> lock(g_host_mutex);
-    for (HostContext &c : g_host_context[dev]) c.destroy();
-    g_host_context[dev].clear();
+    KeptContexts &kept = g_host_context[dev];
+    while (kept.n > 0) kept.at[--kept.n].destroy();
     if (g_host_pool[dev]) {
         const cudaError_t e = cudaMemPoolTrimTo(g_host_pool[dev], 0);
         if (e != cudaSuccess)

@@ -111,3 +111,27 @@ def test_scratch_is_given_back(zipvl):
         from_the_host(zipvl, x, 0.9)
         zipvl.zipvl_release_host_scratch()
         assert torch.cuda.mem_get_info()[0] >= before - (2 << 20)      # (the scratch is some 150 MB)
+
+
+def test_more_calls_at_once_than_are_kept(zipvl):
+    """Eight threads at a time, of which the library keeps the streams of four: the others' are made and destroyed."""
+    x = inputs(700, 4, 4, 64, torch.bfloat16, 3)
+    want, got = on_the_device(zipvl, x, 0.9), []
+    gate = threading.Barrier(8)
+
+    def work():
+        torch.cuda.set_device(0)
+        for _ in range(3):
+            gate.wait(60)
+            got.append(from_the_host(zipvl, x, 0.9))
+
+    threads = [threading.Thread(target=work) for _ in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert len(got) == 24
+    for r in got:
+        same(r, want)
+    zipvl.zipvl_release_host_scratch()
+    same(from_the_host(zipvl, x, 0.9), want)
