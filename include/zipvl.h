@@ -94,7 +94,9 @@ uint64_t zipvl_launch_count(void);
 
 /* Bytes of device workspace `op` needs for this layer.  `n_probe` matters to
  * SCORE only; for DECODE pass the batch size in `batch` and the largest cache
- * length any request can reach in layer->L.  Returns 0 on a bad argument. */
+ * length any request can reach in layer->L.  The answer never falls as L, n_probe
+ * or batch grow, so a workspace for the largest call serves every smaller one.
+ * Returns 0 on a bad argument. */
 size_t zipvl_workspace_bytes(int32_t op, const zipvl_layer *layer, int32_t n_probe, int32_t batch);
 
 /*

@@ -251,7 +251,7 @@ zipvl_status zipvl_decode(const zipvl_decode_desc *d, const void *q, const void 
         return fail(ZIPVL_ERR_INVALID_ARG, "zipvl_decode: softmax_scale");
     if (!aligned16(q) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(out) || !aligned16(ws))
         return fail(ZIPVL_ERR_INVALID_ARG, "zipvl_decode: tensors must be 16-byte aligned");
-    const size_t need = align256(decode_ws_bytes(d->batch, d->n_q_heads, d->head_dim, max_len, d->n_kv_heads, d->dtype));
+    const size_t need = align256(decode_ws_need(d->batch, d->n_q_heads, d->head_dim, max_len, d->n_kv_heads, d->dtype));
     if (ws_bytes < need) return fail(ZIPVL_ERR_WORKSPACE, "zipvl_decode: workspace %zu < %zu", ws_bytes, need);
     const float scale = d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / sqrtf((float)d->head_dim);
     return launch_decode(*d, scale * kLog2e, q, k_new, v_new, k_cache, v_cache, cache_off, capacity,

@@ -179,9 +179,12 @@ struct PageArgs {
     int stride, shift, n_pages;
 };
 
-// (Hkv and dtype decide whether the grouped-query tensor-core kernel may run: 0 / -1 = it may not)
-size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv = 0, int dtype = -1);
-// workspace of the decode over the mixed-precision cache (kvquant_decode.cu)
+// What a step needs, and (decode_ws_bytes) a bound that no smaller batch or length exceeds: zipvl_workspace_bytes answers with
+// that, so a workspace sized for the largest step serves every other.
+size_t decode_ws_need(int B, int Hq, int D, int max_len, int Hkv, int dtype);
+size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv, int dtype);
+// the same for the decode over the mixed-precision cache (kvquant_decode.cu)
+size_t decode_quant_ws_need(int B, int Hq, int Hkv, int D, int max_len);
 size_t decode_quant_ws_bytes(int B, int Hq, int Hkv, int D, int max_len);
 // caches != nullptr: the new length of request b goes to caches[b].lens[0] instead of seq_lens[b].
 zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int n_chunks, const float *ws,
@@ -191,6 +194,7 @@ zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int n_chunks, 
 // 32 query heads per kv head.  partials, lens: pieces of the workspace (decode.cu).
 bool decode_mma_supported(const zipvl_decode_desc &d);
 int decode_mma_chunk(int B, int Hq, int Hkv, int D, int max_len);
+size_t decode_mma_slots(int B, int Hq, int Hkv, int D, int max_len);
 zipvl_status launch_decode_mma(const zipvl_decode_desc &d, float scale_log2, const void *q, const void *k_new,
                                const void *v_new, void *k_cache, void *v_cache, const int64_t *cache_off, PageArgs pg,
                                const int32_t *capacity, int32_t *seq_lens, int max_len, float *partials, int *lens, void *out,

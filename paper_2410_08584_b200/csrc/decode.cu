@@ -443,11 +443,18 @@ zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int n_chunks, 
     return ZIPVL_OK;
 }
 
-size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv, int dtype) {
+size_t decode_ws_need(int B, int Hq, int D, int max_len, int Hkv, int dtype) {
     // (a shape of the tensor-core kernel may be sent to the CUDA-core one, see dispatch_decode)
     const size_t simt = partial_bytes(B, Hq, D, max_len, decode_chunk(B, Hq, max_len));
     const size_t mma = mma_shape(Hq, Hkv, D, dtype) ? partial_bytes(B, Hq, D, max_len, decode_mma_chunk(B, Hq, Hkv, D, max_len)) : 0;
     return std::max(simt, mma) + length_bytes(B);
+}
+size_t decode_ws_bytes(int B, int Hq, int D, int max_len, int Hkv, int dtype) {
+    // CUDA-core chunks: 32 to 512 rows, between them as many as make eight CTAs per SM (or one per request and head)
+    const auto cut = [&](size_t rows) { return (size_t)B * Hq * ((max_len + rows - 1) / rows); };
+    const size_t simt = std::max(cut(512), std::min(cut(32), (size_t)148 * 8 + (size_t)B * Hq));
+    const size_t mma = mma_shape(Hq, Hkv, D, dtype) ? decode_mma_slots(B, Hq, Hkv, D, max_len) : 0;
+    return align256(std::max(simt, mma) * (D + 2) * sizeof(float)) + length_bytes(B);
 }
 
 namespace {
@@ -566,7 +573,7 @@ extern "C" zipvl_status zipvl_decode_noalloc(const zipvl_decode_desc *d, const v
         return fail(ZIPVL_ERR_INVALID_ARG, "%s: softmax_scale", who);
     if (((uintptr_t)q | (uintptr_t)k_cache | (uintptr_t)v_cache | (uintptr_t)out) & 15u)
         return fail(ZIPVL_ERR_INVALID_ARG, "%s: tensors must be 16-byte aligned", who);
-    const size_t need = decode_ws_bytes(d->batch, d->n_q_heads, d->head_dim, max_len, d->n_kv_heads, d->dtype);
+    const size_t need = decode_ws_need(d->batch, d->n_q_heads, d->head_dim, max_len, d->n_kv_heads, d->dtype);
     if (need > kNoAllocScratchBytes)
         return fail(ZIPVL_ERR_WORKSPACE,
                     "%s: batch %d x %d heads x max_len %d needs %zu bytes of scratch, the built-in "
@@ -617,7 +624,7 @@ extern "C" zipvl_status zipvl_decode_paged(const zipvl_decode_desc *d, const voi
         return fail(ZIPVL_ERR_INVALID_ARG, "%s: softmax_scale", who);
     if (((uintptr_t)q | (uintptr_t)k_pages | (uintptr_t)v_pages | (uintptr_t)out | (uintptr_t)ws) & 15u)
         return fail(ZIPVL_ERR_INVALID_ARG, "%s: tensors must be 16-byte aligned", who);
-    const size_t need = (decode_ws_bytes(d->batch, d->n_q_heads, d->head_dim, max_len, d->n_kv_heads, d->dtype) + 255) & ~(size_t)255;
+    const size_t need = (decode_ws_need(d->batch, d->n_q_heads, d->head_dim, max_len, d->n_kv_heads, d->dtype) + 255) & ~(size_t)255;
     if (ws_bytes < need) return fail(ZIPVL_ERR_WORKSPACE, "%s: workspace %zu < %zu", who, ws_bytes, need);
     const float scale = d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / sqrtf((float)d->head_dim);
     return dispatch_decode(*d, scale * kLog2e, q, k_new, v_new, k_pages, v_pages, nullptr,

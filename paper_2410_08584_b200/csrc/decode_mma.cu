@@ -448,6 +448,15 @@ int decode_mma_chunk(int B, int Hq, int Hkv, int D, int max_len) {
     return std::max(std::min(max_rows(Hq / Hkv, D), std::max(64, tiles_of(n))), tiles_of(65535));
 }
 
+// Chunks times query heads of all requests, for this problem or any smaller batch or length: a chunk is no shorter than 64
+// rows or max_rows allow, and in between there are no more of them than one wave (or one per request).
+size_t decode_mma_slots(int B, int Hq, int Hkv, int D, int max_len) {
+    const int G = Hq / Hkv, nt = G == 1 ? 0 : (G + 7) / 8;
+    const auto cut = [&](size_t rows) { return (size_t)B * Hq * ((max_len + rows - 1) / rows); };
+    const size_t wave = (size_t)G * std::max<size_t>(148 * ctas_per_sm(nt, D), (size_t)B * Hkv);
+    return std::max(cut(max_rows(G, D)), std::min(cut(64), wave));
+}
+
 zipvl_status launch_decode_mma(const zipvl_decode_desc &d, float scale_log2, const void *q, const void *k_new,
                                const void *v_new, void *k_cache, void *v_cache, const int64_t *cache_off, PageArgs pg,
                                const int32_t *capacity, int32_t *seq_lens, int max_len, float *partials, int *lens, void *out,

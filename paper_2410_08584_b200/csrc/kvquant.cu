@@ -332,7 +332,7 @@ extern "C" zipvl_status zipvl_decode_quant(const zipvl_decode_desc *d, const voi
     QuantBlocks qb;
     const zipvl_status s = check_blocks(who, d->n_kv_heads, k_hi, v_hi, params_hi, cap_hi, k_lo, v_lo, params_lo, cap_lo, &qb);
     if (s != ZIPVL_OK) return s;
-    const size_t need = (decode_quant_ws_bytes(1, d->n_q_heads, d->n_kv_heads, d->head_dim, max_len) + 255) & ~(size_t)255;
+    const size_t need = (decode_quant_ws_need(1, d->n_q_heads, d->n_kv_heads, d->head_dim, max_len) + 255) & ~(size_t)255;
     if (ws_bytes < need) return fail(ZIPVL_ERR_WORKSPACE, "%s: workspace %zu < %zu", who, ws_bytes, need);
     const float scale = (d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / sqrtf((float)d->head_dim)) * kLog2e;
     return launch_decode_quant(*d, scale, q, k_new, v_new, qb, lens, nullptr, max_len, out, ws, status_word,
@@ -349,7 +349,7 @@ extern "C" zipvl_status zipvl_decode_quant_batch(const zipvl_decode_desc *d, con
     if (d->batch < 1 || d->batch > 65535) return fail(ZIPVL_ERR_INVALID_ARG, "%s: batch %d not in [1, 65535]", who, d->batch);
     if (d->n_kv_heads > 1024 / 16) return fail(ZIPVL_ERR_UNSUPPORTED, "%s: more than 64 KV heads", who);
     if (!caches || ((uintptr_t)caches & 7u)) return fail(ZIPVL_ERR_INVALID_ARG, "%s: caches is NULL or misaligned", who);
-    const size_t need = (decode_quant_ws_bytes(d->batch, d->n_q_heads, d->n_kv_heads, d->head_dim, max_len) + 255) & ~(size_t)255;
+    const size_t need = (decode_quant_ws_need(d->batch, d->n_q_heads, d->n_kv_heads, d->head_dim, max_len) + 255) & ~(size_t)255;
     if (ws_bytes < need) return fail(ZIPVL_ERR_WORKSPACE, "%s: workspace %zu < %zu", who, ws_bytes, need);
     const float scale = (d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / sqrtf((float)d->head_dim)) * kLog2e;
     return launch_decode_quant(*d, scale, q, k_new, v_new, QuantBlocks{}, nullptr, caches, max_len, out, ws, status_word,

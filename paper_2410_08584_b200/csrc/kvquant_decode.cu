@@ -484,8 +484,13 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
 // a larger batch is ragged, and cutting it one and a half times as fine keeps the SMs busy when the
 // shorter requests leave their last chunks empty (6 requests of 1.4K-5.9K rows: 142 -> 119 us for four layers).
 int quant_chunk(int B, int Hkv, int max_len) {
-    const long long rows = (long long)B * Hkv * max_len / (148 * (B <= 3 ? 14 : 24));
+    const long long warps = 148 * (B <= 3 ? 14 : 24), rows = ((long long)B * Hkv * max_len + warps - 1) / warps;
     return (int)std::min<long long>(512, std::max<long long>(32, (rows + 31) / 32 * 32));
+}
+// Chunks times query heads of all requests, for this problem or any smaller batch or length (see quant_chunk)
+size_t quant_slots(int B, int Hq, int Hkv, int max_len) {
+    const auto cut = [&](size_t rows) { return (size_t)B * Hq * ((max_len + rows - 1) / rows); };
+    return std::max(cut(512), std::min(cut(32), (size_t)(Hq / Hkv) * 148 * (B <= 3 ? 14 : 24) + (size_t)B * Hq));
 }
 size_t quant_partial_bytes(int B, int Hq, int Hkv, int D, int max_len) {
     const int chunk = quant_chunk(B, Hkv, max_len);
@@ -528,8 +533,11 @@ zipvl_status launch_decode_quant(const zipvl_decode_desc &d, float scale_log2, c
 
 }  // namespace kvq
 
-size_t decode_quant_ws_bytes(int B, int Hq, int Hkv, int D, int max_len) {
+size_t decode_quant_ws_need(int B, int Hq, int Hkv, int D, int max_len) {
     return kvq::quant_partial_bytes(B, Hq, Hkv, D, max_len) + (size_t)2 * B * sizeof(int);
+}
+size_t decode_quant_ws_bytes(int B, int Hq, int Hkv, int D, int max_len) {
+    return align256(kvq::quant_slots(B, Hq, Hkv, max_len) * (D + 2) * sizeof(float)) + (size_t)2 * B * sizeof(int);
 }
 
 }  // namespace zipvl

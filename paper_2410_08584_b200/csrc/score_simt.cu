@@ -381,15 +381,19 @@ __global__ void sum_to_double_kernel(int L, const float *__restrict__ x, double 
     if (threadIdx.x == 0) *out = sh[0];
 }
 
-static bool use_cluster(int L, int P) { return L <= 8 * kClusterKeys && P <= 128; }
+constexpr int kClMaxProbes = 128;
+static bool use_cluster(int L, int P) { return L <= 8 * kClusterKeys && P <= kClMaxProbes; }
 
 size_t score_simt_ws_bytes(int L, int Hq, int P) {
     const size_t n_chunks = (L + kChunk - 1) / kChunk;
     size_t stats = (size_t)Hq * n_chunks * P * sizeof(float2);
     stats = (stats + 255) & ~(size_t)255;
-    const size_t cluster = (size_t)Hq * ((P + kClProbes - 1) / kClProbes) * L * sizeof(float);
+    // Room for every shorter row and smaller number of probes too: a buffer sized for the largest serves all.  The
+    // one-sweep kernels need most at their own limits and nothing beyond.
+    const int cl = L < 8 * kClusterKeys ? L : 8 * kClusterKeys, cp = P < kClMaxProbes ? P : kClMaxProbes;
+    const size_t cluster = (size_t)Hq * ((cp + kClProbes - 1) / kClProbes) * cl * sizeof(float);
     const size_t two_pass = stats + (size_t)Hq * L * sizeof(float);
-    return use_cluster(L, P) && cluster > two_pass ? cluster : two_pass;
+    return cluster > two_pass ? cluster : two_pass;
 }
 
 template <int D, int NS>

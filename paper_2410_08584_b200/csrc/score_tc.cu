@@ -18,6 +18,8 @@
 // Every head adds its column sums to 64-bit fixed-point totals (integer adds: no order to
 // depend on, so results repeat bit for bit); the last CTA to finish a key chunk turns the
 // totals into floats and normalises.
+#include <algorithm>
+
 #include <cuda.h>
 
 #include "tc.cuh"
@@ -420,11 +422,10 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
+constexpr int kResident = 2 * 148;   // CTAs of a launch: all resident at once, two per SM
 int tiles_per_chunk_for(int L, int Hq) {
-    // all CTAs of a launch are resident at once: two per SM on 148 SMs, so at most
-    // 296 / Hq key chunks per head
     const int n_tiles = (L + kTile - 1) / kTile;
-    const int max_chunks = (Hq >= 296) ? 1 : 296 / Hq;
+    const int max_chunks = (Hq >= kResident) ? 1 : kResident / Hq;
     int tpc = (n_tiles + max_chunks - 1) / max_chunks;
     if (tpc < 1) tpc = 1;
     return tpc;
@@ -441,14 +442,13 @@ bool score_tc_supported(const LayerArgs &a, int dtype, int n_probe) {
 }
 
 size_t score_tc_ws_bytes(int L, int Hq, int, int, int n_seq) {
-    const int n_tiles = (L + kTile - 1) / kTile;
-    const int tpc = tiles_per_chunk_for(L, Hq * n_seq);
-    const size_t n_chunks = (n_tiles + tpc - 1) / tpc;
-    size_t stats = (size_t)Hq * n_chunks * kMaxProbe * sizeof(float2);
-    stats = (stats + 255) & ~(size_t)255;
-    stats = ((stats * n_seq) + 255) & ~(size_t)255;
+    // Room for every shorter row and smaller batch too, whose chunks may be more: there are at most as many chunks as
+    // tiles, and in all heads at most kResident unless every head has one.
+    const size_t n_tiles = (L + kTile - 1) / kTile, heads = (size_t)Hq * n_seq;
+    const auto chunks = [&](size_t rows) { return std::min(rows * n_tiles, std::max<size_t>(kResident, rows)); };
+    const size_t stats = (chunks(heads) * kMaxProbe * sizeof(float2) + 255) & ~(size_t)255;
     const size_t totals = ((size_t)n_seq * L * sizeof(unsigned long long) + 255) & ~(size_t)255;
-    return stats + totals + n_seq * n_chunks * sizeof(int);
+    return stats + totals + chunks(n_seq) * sizeof(int);
 }
 
 zipvl_status launch_score_tc(const LayerArgs &a, const void *q, const void *k,
