@@ -469,7 +469,7 @@ zipvl_status zipvl_release_host_scratch(void);
 /*
  * zipvl_selftest_wait_timeout -- run a bounded device wait out, on purpose and harmlessly.
  * (No counterpart in the paper: a check of the library's own failure handling.)
- * Every wait inside the tensor-core kernels gives up after a fixed number of polls, raises
+ * Every wait inside the tensor-core kernels gives up after a second and a half (or 2^24 polls), raises
  * its thread block's abort flag, lets all warps leave through the common exit and reports
  * ZIPVL_DEV_TIMEOUT.  This call launches one 128-thread block that uses that same wait:
  * warp 0 waits on a barrier that completes, warps 1-3 on one that nobody arrives at, each

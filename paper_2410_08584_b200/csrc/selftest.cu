@@ -1,6 +1,6 @@
 // Self-test of the bounded device waits.  Every wait inside the tensor-core kernels
 // (on an mbarrier that a TMA copy, an async copy group or a tcgen05.commit completes)
-// goes through ptx::mbar_wait, which gives up after a fixed number of polls, raises the
+// goes through ptx::mbar_wait, which gives up after a fixed number of polls or a second and a half, raises the
 // CTA's abort flag and lets every role unwind to the common exit, where the flag becomes
 // ZIPVL_DEV_TIMEOUT in the caller's status word.  Nothing in the library can make such a
 // wait run out on purpose, so this file holds a kernel that can: one CTA whose warps wait,

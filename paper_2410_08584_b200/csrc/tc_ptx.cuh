@@ -37,14 +37,28 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait: gives up after `limit` polls and returns false (the caller
-// records ZIPVL_DEV_TIMEOUT and unwinds); never spins forever.
-constexpr uint32_t kWaitLimit = 1u << 24;
+__device__ __forceinline__ uint32_t clock_ns() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
+    return t;
+}
+// Bounded wait: gives up after `limit` polls or kWaitNs, whichever comes first, and returns false (the
+// caller records ZIPVL_DEV_TIMEOUT and unwinds); never spins forever.  A poll suspends the thread for up to
+// 4 us, so a number of polls alone is no bound anybody would notice: 2^24 of them take 67 seconds.  The longest wait
+// of a call that runs is its own length, some milliseconds.  The time is looked at once a millisecond, the flag behind the first poll too (a
+// role that unwinds meets one wait per tile).
+constexpr uint32_t kWaitLimit = 1u << 24, kWaitNs = 1500000000u;
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                           uint32_t limit = kWaitLimit) {
+    uint32_t start = 0;
     for (uint32_t it = 0; it < limit; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 1023u) == 1023u && *abort_flag) return false;
+        if ((it & 255u) == 0u && *abort_flag) return false;
+        if ((it & 255u) == 255u) {
+            const uint32_t now = clock_ns();
+            if (it == 255u) start = now;
+            else if (now - start > kWaitNs) break;
+        }
     }
     *abort_flag = 1;
     return false;
