@@ -405,6 +405,23 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
             // late: a step of both tiles went from 4050 to 3620 cycles.  It needs the first and the
             // diagonal tile to take no longer than the others (see the mask below): the other tile waits for them.
             // Sleeping on one tile with a time limit and looking at the other was slower than polling.
+            //
+            // Why no wait here can miss its phase or wait for itself (seq: K0 V0 K1 V1 ... in the ring of five slots):
+            //   - a parity says "done" also two phases early, so whoever waits for a phase must know that the one
+            //     before it is over.  This warp looks at `full` of K(n+1) = seq 2n+2 (and of the last V) only.
+            //     The phase before in that slot is seq 2n-3; the step before waited for seq 2n, every producer
+            //     thread announces in order, so 2n-3 is over.  It cannot be a phase late either: slot 2n+2 is filled
+            //     again only after release(2n+2), which the later user (B, if it uses the slot) issues below its wait;
+            //   - a producer thread waits for `empty` of the slot it filled last itself, and the next release of that
+            //     slot needs its own announcement: never more than one phase apart;
+            //   - p_full[x], s_full[x]: one waiting role each, which sees every phase; S(n+1) is issued behind the wait
+            //     for P(n), P(n+1) follows S(n+1);
+            //   - progress: K(n+1) goes into the slot of seq 2n-3, released behind B(n-2)'s MMAs, all issued before this
+            //     wait.  P(n) needs S(n) of its own tile only, issued a step ago.  The order of the tiles is no
+            //     condition of either, so neither tile waits for a step that is issued behind it;
+            //   - all of it takes one n_valid per CTA.  Every thread reads *k_dev for itself, so the read must stay
+            //     behind the dependency wait (see redefine_pointer): a CTA that was staged early could see the count
+            //     before and after the selection wrote it, in different warps, and its roles would count differently.
             // The later user of a ring slot, B if it uses the slot at all, releases it.
             const int cnt[2] = {n_a, has_b ? n_kv : 0};
             bool ok = !*abort_flag;
@@ -469,17 +486,11 @@ prefill_tc_kernel(LayerArgs a, const __nv_bfloat16 *__restrict__ q,
                 // On the diagonal tile row r sees columns 0..r.  A warp's 32 rows share their
                 // 32-column chunk: chunks below it are fully visible, the chunk with the
                 // warp's own index is cut per lane (column e <= lane), chunks above it are
-                // fully masked.  The masked scores become -inf here and the rest is the code of every
-                // other tile: a second copy of the softmax for the diagonal would run cold once per
-                // CTA (3000 cycles for half a tile's work).
-                // On the diagonal tile row r sees columns 0..r.  A warp's 32 rows share their
-                // 32-column chunk: chunks below it are fully visible, the chunk with the
-                // warp's own index is cut per lane (column e <= lane), chunks above it are
                 // fully masked.  The masked scores become -inf here and the rest is the code of every other
                 // tile.  A softmax of its own for the diagonal, without the masked exponentials, ran cold once
-                // per CTA: 3000 cycles for half a tile's work (together with the order of the issuer: 2944
-                // tokens, 32 heads, whole layer 104.9 -> 99.1 us, 7181 tokens 323 -> 305, 18432 with 28 heads
-                // on 4 2090 -> 2050; the loop body must stay small, a test per chunk inside it cost 2%).
+                // per CTA: 3000 cycles for half a tile's work (together with the order of the issuer and the
+                // announcement of the tail: 2944 tokens, 32 heads, whole layer 102.25 -> 96.50 us, 18432 with 28 heads
+                // on 4 2181 -> 2121; the loop body must stay small, a test per chunk inside it cost 2%).
                 if (__builtin_expect(n == diag_tile, 0)) {
                     tmem_wait_ld();
 #pragma unroll
