@@ -31,6 +31,10 @@
 //   - K of the warp's next tile is fetched as soon as S is computed, V as soon as O is: 16 loads of 16
 //     bytes per lane in flight.  The warps of a CTA take every fourth tile of its chunk and are merged
 //     through shared memory at the end; the chunks by decode_merge_kernel.
+//   - more than eight heads: two to four tiles of eight, whose chains, votes and merges run side by side.  Two
+//     CTAs fit an SM then, and from 25 heads of 128 channels on their eight warps no longer hide each other's
+//     latencies (issue slots 31% busy, tensor pipe 23%): 64 requests of 10K-20K rows on 2 kv heads, 24 heads 187 us
+//     (5.3 TB/s), 34 heads 212, 64 heads 273.
 // Grid x is the kv head: the CTAs of one chunk run side by side and read whole rows of the cache together.
 // A tile is 16 rows, chunks start at multiples of 16 and pages are at least 16 rows, so a paged
 // cache costs one table look-up per tile.
@@ -44,9 +48,11 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kWarps = 4;
+constexpr int kWarps = 4;         // (and of head tiles at most: each warp brings one into shared memory)
 // rows of a CTA: the fewer CTAs share a row (kv heads), the more a partial weighs against the rows behind it
-constexpr int max_rows(int G, int D) { return D == 64 ? 768 : G == 1 ? 1024 : 1536; }
+// (more than eight heads: from 512 on, see decode_mma_chunk)
+constexpr int max_rows(int G, int D) { return G > 8 ? 1536 : D == 64 ? 768 : G == 1 ? 1024 : 1536; }
+constexpr int min_large(int G, int D) { return G > 8 ? 512 : max_rows(G, D); }
 // (their registers; NT = 0: one query head per kv head)
 __host__ __device__ constexpr int ctas_per_sm(int NT, int D) { return NT > 1 ? 2 : D == 64 ? 6 : 3; }
 
@@ -124,8 +130,9 @@ decode_mma_kernel(DmArgs a) {
     constexpr float kGrow = kHalf ? 8.f : 32.f;
     // the three parts of a single head's weight, of eight bits each: multiplied up in IEEE half
     constexpr float kTop = kHalf ? 128.f : 1.f, kStep = kHalf ? 256.f : 1.f;
-    __shared__ float sm_o[kWarps][8][D];
-    __shared__ float sm_m[kWarps][8], sm_l[kWarps][8];
+    constexpr int ET = NT > 1 ? 2 : 1;               // head tiles merged at a time
+    __shared__ float sm_o[kWarps][8 * ET][D];
+    __shared__ float sm_m[kWarps][8 * ET], sm_l[kWarps][8 * ET];
     __shared__ uint4 sm_q[NT > 2 ? NT * 8 * (D / 8) : 1];
 
     grid_launch_dependents();
@@ -146,9 +153,9 @@ decode_mma_kernel(DmArgs a) {
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
             for (int j = 0; j < KJ; ++j) qr[NT > 2 ? 0 : nt][j] = q_piece(nt, j);
-    } else if (warp == 0) {
-        for (int nt = 0; nt < NT; ++nt)
-            for (int j = 0; j < KJ; ++j) sm_q[(nt * KJ + j) * 32 + lane] = q_piece(nt, j);
+    } else if (warp < NT) {
+#pragma unroll
+        for (int j = 0; j < KJ; ++j) sm_q[(warp * KJ + j) * 32 + lane] = q_piece(warp, j);
     }
 
     // A request whose length is negative or beyond its capacity, or whose cache offset breaks the
@@ -178,8 +185,6 @@ decode_mma_kernel(DmArgs a) {
         }
         return;
     }
-    if (NT > 2) __syncthreads();
-
     const int new_row = appended ? old_len : -1;     // (== len when max_len cuts it off: never loaded)
     const long long pitch = (long long)a.Hkv * RB;
     const char *kb = a.k_cache + coff + (long long)hkv * RB, *vb = a.v_cache + coff + (long long)hkv * RB;
@@ -236,6 +241,7 @@ decode_mma_kernel(DmArgs a) {
         load_k(base, off);
         load_v(base, off);
     }
+    if (NT > 2) __syncthreads();                     // the query heads are in shared memory
     for (; base < c1; base += kWarps * 16, off = next_off) {
         const bool more = base + kWarps * 16 < c1;
         next_off = more ? tile_off(base + kWarps * 16) : -1;
@@ -263,11 +269,13 @@ decode_mma_kernel(DmArgs a) {
         }
         float c[NT][4];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
             for (int e = 0; e < 4; ++e) c[nt][e] = 0.f;
 #pragma unroll
-            for (int j = 0; j < KJ; ++j) {
+        for (int j = 0; j < KJ; ++j)                 // (the head tiles' chains side by side)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
                 const uint4 qv = NT > 2 ? sm_q[(nt * KJ + j) * 32 + lane] : qr[NT > 2 ? 0 : nt][j];
                 if (kOne) {
                     float x[4], y[4];
@@ -280,7 +288,6 @@ decode_mma_kernel(DmArgs a) {
                 mma16<kHalf>(c[nt], kr[0][j][0], kr[1][j][0], kr[0][j][1], kr[1][j][1], qv.x, qv.y);
                 mma16<kHalf>(c[nt], kr[0][j][2], kr[1][j][2], kr[0][j][3], kr[1][j][3], qv.z, qv.w);
             }
-        }
         if (more) load_k(base + kWarps * 16, next_off);
         if (off < 0) {                               // (uniform)
             if (more) load_v(base + kWarps * 16, next_off);
@@ -288,13 +295,17 @@ decode_mma_kernel(DmArgs a) {
         }
         // ---- weights of rows g and g + 8 for heads 2 t and 2 t + 1
         uint32_t pb[NT][2];
+        bool grow = false;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) c[nt][e] = (g + 8 * (e >> 1) < rows) ? c[nt][e] * a.scale_log2 : -INFINITY;
-            const float mx0 = fmaxf(c[nt][0], c[nt][2]), mx1 = fmaxf(c[nt][1], c[nt][3]);
-            if (__any_sync(0xffffffffu, mx0 > m[nt][0] + kGrow || mx1 > m[nt][1] + kGrow)) {
-                float mx[2] = {mx0, mx1}, f[2];
+            grow |= fmaxf(c[nt][0], c[nt][2]) > m[nt][0] + kGrow || fmaxf(c[nt][1], c[nt][3]) > m[nt][1] + kGrow;
+        }
+        if (__any_sync(0xffffffffu, grow)) {         // (one vote for all head tiles: between two of them nothing waits)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                float mx[2] = {fmaxf(c[nt][0], c[nt][2]), fmaxf(c[nt][1], c[nt][3])}, f[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
 #pragma unroll
@@ -307,6 +318,9 @@ decode_mma_kernel(DmArgs a) {
 #pragma unroll
                 for (int s = 0; s < VS; ++s) { o[nt][s][0] *= f[0]; o[nt][s][1] *= f[1]; o[nt][s][2] *= f[0]; o[nt][s][3] *= f[1]; }
             }
+        }
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
             const float r0 = m[nt][0] == -INFINITY ? 0.f : m[nt][0], r1 = m[nt][1] == -INFINITY ? 0.f : m[nt][1];
             if (kOne) {
                 // every column holds the one head: columns 0, 1, 2 take the three parts of its weight
@@ -323,9 +337,14 @@ decode_mma_kernel(DmArgs a) {
             const float p2 = fast_exp2(c[nt][2] - r0), p3 = fast_exp2(c[nt][3] - r1);
             l[nt][0] += p0 + p2;
             l[nt][1] += p1 + p3;
-            pb[nt][0] = transpose8(pack16<kHalf>(p0, p1));
-            pb[nt][1] = transpose8(pack16<kHalf>(p2, p3));
+            c[nt][0] = p0; c[nt][1] = p1; c[nt][2] = p2; c[nt][3] = p3;
         }
+        if (!kOne)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                pb[nt][0] = transpose8(pack16<kHalf>(c[nt][0], c[nt][1]));
+                pb[nt][1] = transpose8(pack16<kHalf>(c[nt][2], c[nt][3]));
+            }
 #pragma unroll
         for (int j = 0; j < VJ; ++j)
 #pragma unroll
@@ -365,21 +384,24 @@ decode_mma_kernel(DmArgs a) {
             }
     }
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-        if (nt > 0) __syncthreads();
+    for (int nt0 = 0; nt0 < NT; nt0 += ET) {
+        if (nt0 > 0) __syncthreads();
 #pragma unroll
-        for (int h = 0; h < (kOne ? 1 : 2); ++h) {
+        for (int nt = nt0; nt < (nt0 + ET < NT ? nt0 + ET : NT); ++nt)
 #pragma unroll
-            for (int x = 4; x < 32; x <<= 1) l[nt][h] += __shfl_xor_sync(0xffffffffu, l[nt][h], x);
-            if (kOne && t > 0) continue;
-            if (g == 0) { sm_m[warp][2 * t + h] = m[nt][h]; sm_l[warp][2 * t + h] = l[nt][h]; }
+            for (int h = 0; h < (kOne ? 1 : 2); ++h) {
 #pragma unroll
-            for (int s = 0; s < VS; ++s) {
-                *reinterpret_cast<float2 *>(&sm_o[warp][2 * t + h][channel(s)]) = make_float2(o[nt][s][h], o[nt][s][2 + h]);
+                for (int x = 4; x < 32; x <<= 1) l[nt][h] += __shfl_xor_sync(0xffffffffu, l[nt][h], x);
+                if (kOne && t > 0) continue;
+                const int at = (nt - nt0) * 8 + 2 * t + h;
+                if (g == 0) { sm_m[warp][at] = m[nt][h]; sm_l[warp][at] = l[nt][h]; }
+#pragma unroll
+                for (int s = 0; s < VS; ++s)
+                    *reinterpret_cast<float2 *>(&sm_o[warp][at][channel(s)]) = make_float2(o[nt][s][h], o[nt][s][2 + h]);
             }
-        }
         __syncthreads();
-        const int n_heads = min(8, G - nt * 8);
+        const int n_heads = min(8 * ET, G - nt0 * 8);
+#pragma unroll(NT > 1 ? 2 : 1)
         for (int e = threadIdx.x; e < n_heads * (D / 2); e += kWarps * 32) {
             const int h = e / (D / 2), ch = 2 * (e % (D / 2));
             float M = -INFINITY, L = 0.f, x = 0.f, y = 0.f;
@@ -403,7 +425,7 @@ decode_mma_kernel(DmArgs a) {
                 if (!(fabsf(u) < INFINITY)) x = u;
                 if (!(fabsf(v) < INFINITY)) y = v;
             }
-            float *p = dst + (nt * 8 + h) * head_pitch;
+            float *p = dst + (nt0 * 8 + h) * head_pitch;
             *reinterpret_cast<float2 *>(p + 2 + ch) = make_float2(x, y);
             if (ch == 0) *reinterpret_cast<float2 *>(p) = make_float2(M, L);
         }
@@ -419,7 +441,8 @@ cudaError_t launch(const DmArgs &a, int B, cudaStream_t st) {
 template <bool kHalf, int D>
 cudaError_t launch(const DmArgs &a, int B, cudaStream_t st) {
     const int G = a.Hq / a.Hkv;
-    return G == 1 ? launch<kHalf, D, 0>(a, B, st) : G <= 8 ? launch<kHalf, D, 1>(a, B, st) : G <= 16 ? launch<kHalf, D, 2>(a, B, st) : launch<kHalf, D, 4>(a, B, st);
+    return G == 1 ? launch<kHalf, D, 0>(a, B, st) : G <= 8 ? launch<kHalf, D, 1>(a, B, st) : G <= 16 ? launch<kHalf, D, 2>(a, B, st)
+         : G <= 24 ? launch<kHalf, D, 3>(a, B, st) : launch<kHalf, D, 4>(a, B, st);
 }
 template <bool kHalf>
 cudaError_t launch(const DmArgs &a, int B, int D, cudaStream_t st) {
@@ -444,8 +467,13 @@ int decode_mma_chunk(int B, int Hq, int Hkv, int D, int max_len) {
     const long long groups = (long long)B * Hkv, wave = 148 * ctas_per_sm(nt, D);
     const int n = (int)std::max(1ll, wave / groups);
     const auto tiles_of = [&](long long parts) { return (int)((max_len + parts - 1) / parts + 63) / 64 * 64; };
+    // More than eight heads: an SM holds half the warps and a CTA's set-up and end weigh more, so a last wave that is nearly
+    // empty costs most; six waves at least, in CTAs of 512 rows at least (16 requests of 10K-20K rows, 24 heads on 2: 1536 rows 72.5 us,
+    // 768 62.7, 512 61.1, 384 64.8; 64 such requests, six waves of 1536 rows: 189.0, 189.6, 197.5, 214).
+    const int G = Hq / Hkv, least = min_large(G, D), most = max_rows(G, D);
+    const int large = G > 8 ? std::min(most, std::max(least, (int)(((groups * max_len) / (6 * wave) + 63) / 64 * 64))) : most;
     // (the last term: chunks are the grid's y, which ends at 65535)
-    return std::max(std::min(max_rows(Hq / Hkv, D), std::max(64, tiles_of(n))), tiles_of(65535));
+    return std::max(std::min(large, std::max(64, tiles_of(n))), tiles_of(65535));
 }
 
 // Chunks times query heads of all requests, for this problem or any smaller batch or length: a chunk is no shorter than 64
@@ -454,7 +482,7 @@ size_t decode_mma_slots(int B, int Hq, int Hkv, int D, int max_len) {
     const int G = Hq / Hkv, nt = G == 1 ? 0 : (G + 7) / 8;
     const auto cut = [&](size_t rows) { return (size_t)B * Hq * ((max_len + rows - 1) / rows); };
     const size_t wave = (size_t)G * std::max<size_t>(148 * ctas_per_sm(nt, D), (size_t)B * Hkv);
-    return std::max(cut(max_rows(G, D)), std::min(cut(64), wave));
+    return std::max(cut(min_large(G, D)), std::min(cut(64), wave));
 }
 
 zipvl_status launch_decode_mma(const zipvl_decode_desc &d, float scale_log2, const void *q, const void *k_new,

@@ -1,0 +1,64 @@
+"""Decode over grouped query heads at the edges of the kernel's head tiles (8, 16, 24 and 32 heads), on contiguous and paged
+caches, with appends, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from parity import check_attention, to_np
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+CODE = {torch.bfloat16: 0, torch.float32: 1, torch.float16: 2}
+
+
+def check_steps(z, lens, Hq, Hkv, d, dtype, page, steps=2, seed=0):
+    """Steps with an appended row each, on a paged cache (pages in random order) or a contiguous one."""
+    g = torch.Generator().manual_seed(seed + Hq + d)
+    B, row = len(lens), Hkv * d
+    caps = [-(-(n + steps) // (page or 1)) * (page or 1) for n in lens]
+    off = np.concatenate([[0], np.cumsum([c * row for c in caps[:-1]])]).astype(np.int64)
+    kc, vc = (torch.randn(sum(caps) * row, generator=g).to(dtype) for _ in range(2))
+    ko, vo, seqo = to_np(kc).copy(), to_np(vc).copy(), np.array(lens, np.int32)
+    desc = z.zipvl_decode_desc(B, Hq, Hkv, d, CODE[dtype], 0.0)
+    seq, cap = torch.tensor(lens, dtype=torch.int32, device=DEV), torch.tensor(caps, dtype=torch.int32, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    if page:
+        n_pages = sum(caps) // page
+        where = torch.randperm(n_pages, generator=g)             # page i of the contiguous layout -> its place in the pool
+        pools = []
+        for c in (kc, vc):
+            pool = torch.empty_like(c).view(n_pages, page, Hkv, d)
+            pool[where] = c.view(n_pages, page, Hkv, d)
+            pools.append(pool.to(DEV))
+        table = torch.zeros(B, max(caps) // page, dtype=torch.int32)
+        at = 0
+        for b, c in enumerate(caps):
+            table[b, :c // page] = where[at:at + c // page].to(torch.int32)
+            at += c // page
+        table = table.to(DEV)
+    else:
+        kd, vd, offd = kc.to(DEV), vc.to(DEV), torch.from_numpy(off).to(DEV)
+    for _ in range(steps):
+        q = torch.randn(B, Hq, d, generator=g).to(dtype)
+        kn, vn = (torch.randn(B, Hkv, d, generator=g).to(dtype) for _ in range(2))
+        if page:
+            out = z.zipvl_decode_paged(desc, q.to(DEV), kn.to(DEV), vn.to(DEV), *pools, table, cap, seq, max(lens) + steps, status=st)
+        else:
+            out = z.zipvl_decode(desc, q.to(DEV), kn.to(DEV), vn.to(DEV), kd, vd, offd, cap, seq, max(lens) + steps, status=st)
+        want = oracle.decode_step(to_np(q), to_np(kn), to_np(vn), ko, vo, off, seqo, Hkv)
+        check_attention(to_np(out), want, dtype)
+    assert st.item() == 0 and np.array_equal(seq.cpu().numpy(), seqo)
+
+
+@pytest.mark.parametrize("G", [8, 9, 16, 17, 24, 25, 32])
+@pytest.mark.parametrize("d,dtype", [(64, torch.float16), (96, torch.bfloat16), (128, torch.bfloat16)])
+@pytest.mark.parametrize("page", [0, 16])
+def test_heads_at_the_edges_of_the_tiles(zipvl, G, d, dtype, page):
+    check_steps(zipvl, [15, 700, 63, 130], 2 * G, 2, d, dtype, page)
+
+
+@pytest.mark.parametrize("G", [9, 17, 32])
+def test_many_heads_on_more_than_a_wave(zipvl, G):
+    """Chunks of 512 rows and more, lengths around their ends."""
+    check_steps(zipvl, [509, 510, 511, 1021, 1022, 1023, 40, 0] * 5, 2 * G, 2, 64, torch.bfloat16, 0, steps=1)
