@@ -301,8 +301,8 @@ zipvl_status zipvl_sparse_prefill_batch(const zipvl_layer *layer, const zipvl_ba
  * Query heads per kv head (Hq / Hkv): up to 8 for any dtype; up to 32 in 16-bit storage.  16-bit
  * storage runs on the tensor cores (the query heads of a kv head are the columns of an MMA, so
  * grouped-query attention stays bound by HBM instead of by multiply-adds), but for contiguous caches
- * of more than three requests with one query head per kv head at head_dim 64, which the CUDA-core
- * kernel serves, as it does fp32.  Same results contract on every path; ZIPVL_DECODE_KERNEL=simt in the
+ * of more than three requests and 100000 or more rows of heads (batch * n_kv_heads * max_len) with one
+ * query head per kv head at head_dim 64, which the CUDA-core kernel serves, as it does fp32.  Same results contract on every path; ZIPVL_DECODE_KERNEL=simt in the
  * environment forces the CUDA-core kernel where it applies.
  */
 zipvl_status zipvl_decode(const zipvl_decode_desc *desc, const void *q, const void *k_new,

@@ -467,14 +467,18 @@ zipvl_status dispatch_decode(const zipvl_decode_desc &d, float scale_log2, const
     // kernel is bound by its multiply-adds (0.49 of the HBM copy rate at four, 0.29 at seven) and
     // reads a row once per eight heads; with one it has too few rows in flight on short caches
     // (one request of 2307 rows: 13.8 against 11.2 us) and too much address arithmetic on
-    // paged ones (26 requests of 560 rows: 57 against 44 us).  It keeps the contiguous caches of many requests
-    // at head_dim 64 (37 requests of 1.3K-3.1K rows: 61 against 64 us).
+    // paged ones (26 requests of 560 rows: 57 against 44 us).  It keeps the contiguous caches at head_dim 64 where there are
+    // more than three requests with 100000 rows of heads or more (B x heads x longest, its time against the other's in us:
+    // 16 x 16 x 700 10.9, 12.5; 16 x 16 x 3000 32.8, 35.3; 64 x 4 x 3000 30.4, 33.5; 64 x 16 x 100 9.0, 9.7; 64 x 16 x 3000
+    // 96.4, 98.7; but 4 x 16 x 3000 12.3, 12.2; 4 x 16 x 700 7.8, 6.1; 16 x 4 x 700 7.0, 6.5; 2 x 16 x 20000 28.9, 26.1; paged
+    // 16 x 16 x 3000 39.5, 36.4).
     // ZIPVL_DECODE_KERNEL=simt in the environment sends shapes of up to eight heads to the CUDA-core kernel
     // all the same (measurements, tests).
     const char *env = getenv("ZIPVL_DECODE_KERNEL");
     const int Hq = d.n_q_heads, Hkv = d.n_kv_heads;
     const bool simt = Hq / Hkv <= 8 && ((env && !strcmp(env, "simt")) ||
-                                        (Hq == Hkv && d.head_dim == 64 && !pg.table && d.batch > 3));
+                                        (Hq == Hkv && d.head_dim == 64 && !pg.table && d.batch > 3 &&
+                                         (long long)d.batch * Hkv * max_len >= 100000));
     if (decode_mma_supported(d) && !simt) {
         const int chunk = decode_mma_chunk(d.batch, Hq, Hkv, d.head_dim, max_len);
         int *lens = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + partial_bytes(d.batch, Hq, d.head_dim, max_len, chunk));

@@ -1,5 +1,5 @@
-"""Decode over grouped query heads at the edges of the kernel's head tiles (8, 16, 24 and 32 heads), on contiguous and paged
-caches, with appends, against the oracle."""
+"""Decode over grouped query heads at the edges of the kernel's head tiles (8, 16, 24 and 32 heads) and over single heads of 64
+channels on either side of the lines between two kernels, on contiguous and paged caches, with appends, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -62,3 +62,11 @@ def test_heads_at_the_edges_of_the_tiles(zipvl, G, d, dtype, page):
 def test_many_heads_on_more_than_a_wave(zipvl, G):
     """Chunks of 512 rows and more, lengths around their ends."""
     check_steps(zipvl, [509, 510, 511, 1021, 1022, 1023, 40, 0] * 5, 2 * G, 2, 64, torch.bfloat16, 0, steps=1)
+
+
+@pytest.mark.parametrize("n,L,H", [(3, 1500, 16), (4, 1500, 16), (4, 1562, 16), (5, 1251, 16), (5, 1240, 16), (4, 63, 3), (7, 20, 1)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("page", [0, 64])
+def test_single_heads_of_64_channels(zipvl, n, L, H, dtype, page):
+    """Either side of the lines between the two kernels: more than three requests, 100000 rows of heads, contiguous."""
+    check_steps(zipvl, [L, 1, 17] + [max(0, L - 7 * i) for i in range(n - 3)], H, H, 64, dtype, page)
