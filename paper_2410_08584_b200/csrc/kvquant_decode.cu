@@ -26,7 +26,8 @@
 //     large has to cancel: the tensor core cuts its sums off instead of rounding them, 2^-23 of the running
 //     sum per MMA.  Error of the fp32 results against 64 bits, N(0, 1) keys and values, queries of four sizes,
 //     1.4K to 9K rows: 0.2 to 0.9 of that of the plain fp32 evaluation that this kernel replaced.
-// A warp owns a chunk of rows of one (request, kv head); the four warps of a CTA take four
+// A warp owns a chunk of rows of one block of one (request, kv head) (a chunk across both blocks pays the set-up and the first
+// loads of either: 1 us of a step of 5); the four warps of a CTA take four
 // neighbouring heads of the same rows (their parameters share 32-byte sectors).  32 rows per step: each
 // lane evaluates the softmax weight of one row (the query repeated over the columns brings a
 // row's score to the lane that needs it), and two more steps are on their way into the warp's own ring.  Nothing is shared between warps: each leaves (m, l, o) for
@@ -426,19 +427,22 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
         lens_ws[2 * b + 1] = room ? 1 : 0;
     }
     if (hkv >= Hkv) return;
-    const int c0 = blockIdx.x * chunk, c1 = min(total, c0 + chunk);
+    // a chunk lies in one block: first those of the 4-bit rows, then those of the 2-bit ones
+    const int rows4 = min(n_hi, total), chunks4 = (rows4 + chunk - 1) / chunk;
+    const bool in4 = (int)blockIdx.x < chunks4;
+    const int r0 = ((int)blockIdx.x - (in4 ? 0 : chunks4)) * chunk, r1 = min(in4 ? rows4 : total - rows4, r0 + chunk);
     float *dst = ws + (((long long)b * Hq + hkv * G) * n_chunks + blockIdx.x) * (D + 2);
     const long long head_pitch = (long long)n_chunks * (D + 2);
     // the appended row belongs to the chunk that ends with it (or, beyond the rows that count, to the last)
     const long long rh = (long long)old_hi * Hkv + hkv;
     NewRow fresh = {k_new + ((long long)b * Hkv + hkv) * D, v_new + ((long long)b * Hkv + hkv) * D, qb.k_hi + rh * (D / 2),
                     qb.v_hi + rh * (D / 2), qb.p_hi + rh * 4};
-    const bool mine = room && old_hi >= c0 && old_hi < c1;
-    if (room && old_hi >= total && (int)blockIdx.x == n_chunks - 1) {
+    const bool mine = room && in4 && old_hi >= r0 && old_hi < r1;
+    if (room && old_hi >= rows4 && (int)blockIdx.x == n_chunks - 1) {
         uint32_t par;
         fresh.quantise<kHalf, D>(lane, par);
     }
-    if (c0 >= c1) {
+    if (r0 >= r1) {
         if (lane < G) {                      // a chunk past the cache: an empty partial
             dst[lane * head_pitch] = -INFINITY;
             dst[lane * head_pitch + 1] = 0.f;
@@ -455,9 +459,10 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
         for (int e = 0; e < 4; ++e) st.o[s][e] = 0.f;
 #pragma unroll
     for (int h = 0; h < NH; ++h) { st.m[h] = -INFINITY; st.m_w[h] = -INFINITY; st.l[h] = 0.f; st.zacc[h] = 0.f; }
-    run_block<4, kHalf, D, G>(st, qb.k_hi, qb.v_hi, qb.p_hi, c0, min(c1, n_hi), Hkv, hkv, qh, scale_log2, ring, lane,
-                              mine ? &fresh : nullptr);
-    run_block<2, kHalf, D, G>(st, qb.k_lo, qb.v_lo, qb.p_lo, max(c0 - n_hi, 0), c1 - n_hi, Hkv, hkv, qh, scale_log2, ring, lane);
+    if (in4)
+        run_block<4, kHalf, D, G>(st, qb.k_hi, qb.v_hi, qb.p_hi, r0, r1, Hkv, hkv, qh, scale_log2, ring, lane, mine ? &fresh : nullptr);
+    else
+        run_block<2, kHalf, D, G>(st, qb.k_lo, qb.v_lo, qb.p_lo, r0, r1, Hkv, hkv, qh, scale_log2, ring, lane);
 
     // ---- this chunk's (m, l, o): o = sum p * (code * v_scale + v_zero).  Lane t < 2 holds the hi parts of
     // heads 2t, 2t + 1, lane t + 2 their lo parts.
@@ -483,18 +488,24 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
 // them even if every request has max_len rows (a few warps of a second wave cost a quarter of a short step);
 // a larger batch is ragged, and cutting it one and a half times as fine keeps the SMs busy when the
 // shorter requests leave their last chunks empty (6 requests of 1.4K-5.9K rows: 142 -> 119 us for four layers).
+// With few heads neither fills the chip, and what counts is the number of partial results to merge: 64 at most
+// (one request of 12000 rows, 4 heads of 64: 13.1 us at 375 chunks, 10.1 at 256, 9.2 at 128 and 64; 6 requests of
+// 12000 rows, one head of 128: 19.1, 14.1, 12.3, 11.8; over 154 shapes 64 is 2% ahead of 128 and 256).
+constexpr int kMaxChunks = 64;
 int quant_chunk(int B, int Hkv, int max_len) {
     const long long warps = 148 * (B <= 3 ? 14 : 24), rows = ((long long)B * Hkv * max_len + warps - 1) / warps;
-    return (int)std::min<long long>(512, std::max<long long>(32, (rows + 31) / 32 * 32));
+    return (int)std::min<long long>(512, std::max<long long>(32, (std::max<long long>(rows, (max_len + kMaxChunks - 1) / kMaxChunks) + 31) / 32 * 32));
 }
+// (one more than the rows fill: either block ends with a part of a chunk)
+int quant_chunks(int max_len, int chunk) { return (max_len + chunk - 1) / chunk + 1; }
 // Chunks times query heads of all requests, for this problem or any smaller batch or length (see quant_chunk)
 size_t quant_slots(int B, int Hq, int Hkv, int max_len) {
     const auto cut = [&](size_t rows) { return (size_t)B * Hq * ((max_len + rows - 1) / rows); };
-    return std::max(cut(512), std::min(cut(32), (size_t)(Hq / Hkv) * 148 * (B <= 3 ? 14 : 24) + (size_t)B * Hq));
+    return std::max(cut(512), std::min(cut(32), (size_t)(Hq / Hkv) * 148 * (B <= 3 ? 14 : 24) + (size_t)B * Hq)) + (size_t)B * Hq;
 }
 size_t quant_partial_bytes(int B, int Hq, int Hkv, int D, int max_len) {
     const int chunk = quant_chunk(B, Hkv, max_len);
-    return ((size_t)B * Hq * ((max_len + chunk - 1) / chunk) * (D + 2) * sizeof(float) + 255) & ~(size_t)255;
+    return align256((size_t)B * Hq * quant_chunks(max_len, chunk) * (D + 2) * sizeof(float));
 }
 
 template <bool kHalf, int D>
@@ -502,7 +513,7 @@ zipvl_status run(const zipvl_decode_desc &d, float scale_log2, const void *q, co
                  const void *v_new, const QuantBlocks &qb, int32_t *lens, const zipvl_quant_cache *caches, int max_len,
                  void *out, void *ws, int32_t *status_word, cudaStream_t st) {
     const int Hq = d.n_q_heads, Hkv = d.n_kv_heads, G = Hq / Hkv, B = d.batch;
-    const int chunk = quant_chunk(B, Hkv, max_len), n_chunks = (max_len + chunk - 1) / chunk;
+    const int chunk = quant_chunk(B, Hkv, max_len), n_chunks = quant_chunks(max_len, chunk);
     float *wsf = reinterpret_cast<float *>(ws);
     int *lens_ws = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + quant_partial_bytes(B, Hq, Hkv, D, max_len));
     auto *kernel = G == 1 ? decode_quant_kernel<kHalf, D, 1> : G == 2 ? decode_quant_kernel<kHalf, D, 2> : decode_quant_kernel<kHalf, D, 4>;
