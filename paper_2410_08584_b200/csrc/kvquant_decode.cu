@@ -484,16 +484,17 @@ decode_quant_kernel(int Hq, int Hkv, float scale_log2, const unsigned short *__r
     }
 }
 
-// Rows per warp, in whole steps.  An SM holds 16 of these warps.  One to three requests: at most one wave of
-// them even if every request has max_len rows (a few warps of a second wave cost a quarter of a short step);
-// a larger batch is ragged, and cutting it one and a half times as fine keeps the SMs busy when the
-// shorter requests leave their last chunks empty (6 requests of 1.4K-5.9K rows: 142 -> 119 us for four layers).
+// Rows per warp, in whole steps.  An SM holds 16 of these warps.  One or two requests: at most one wave of
+// them even if every request has max_len rows; a larger batch is ragged, and cutting it finer keeps the SMs busy when the
+// shorter requests leave their last chunks empty.  24 against 14 warps per SM, the time over nine shapes of three head
+// counts and lengths: 1.00 for one and two requests, 0.95 for three, 0.98, 0.94, 0.93, 0.95 for four, five, six and eight.
 // With few heads neither fills the chip, and what counts is the number of partial results to merge: 64 at most
 // (one request of 12000 rows, 4 heads of 64: 13.1 us at 375 chunks, 10.1 at 256, 9.2 at 128 and 64; 6 requests of
 // 12000 rows, one head of 128: 19.1, 14.1, 12.3, 11.8; over 154 shapes 64 is 2% ahead of 128 and 256).
 constexpr int kMaxChunks = 64;
+constexpr int wave_warps(int B) { return B <= 2 ? 14 : 24; }
 int quant_chunk(int B, int Hkv, int max_len) {
-    const long long warps = 148 * (B <= 3 ? 14 : 24), rows = ((long long)B * Hkv * max_len + warps - 1) / warps;
+    const long long warps = 148 * wave_warps(B), rows = ((long long)B * Hkv * max_len + warps - 1) / warps;
     return (int)std::min<long long>(512, std::max<long long>(32, (std::max<long long>(rows, (max_len + kMaxChunks - 1) / kMaxChunks) + 31) / 32 * 32));
 }
 // (one more than the rows fill: either block ends with a part of a chunk)
@@ -501,7 +502,7 @@ int quant_chunks(int max_len, int chunk) { return (max_len + chunk - 1) / chunk 
 // Chunks times query heads of all requests, for this problem or any smaller batch or length (see quant_chunk)
 size_t quant_slots(int B, int Hq, int Hkv, int max_len) {
     const auto cut = [&](size_t rows) { return (size_t)B * Hq * ((max_len + rows - 1) / rows); };
-    return std::max(cut(512), std::min(cut(32), (size_t)(Hq / Hkv) * 148 * (B <= 3 ? 14 : 24) + (size_t)B * Hq)) + (size_t)B * Hq;
+    return std::max(cut(512), std::min(cut(32), (size_t)(Hq / Hkv) * 148 * wave_warps(B) + (size_t)B * Hq)) + (size_t)B * Hq;
 }
 size_t quant_partial_bytes(int B, int Hq, int Hkv, int D, int max_len) {
     const int chunk = quant_chunk(B, Hkv, max_len);

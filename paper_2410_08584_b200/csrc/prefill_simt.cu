@@ -364,13 +364,17 @@ zipvl_status run(const LayerArgs &a, const void *q, const void *k, const void *v
     if (tiles > 65535) return fail(ZIPVL_ERR_UNSUPPORTED, "sparse_prefill: k_max %d on the CUDA-core path", k_max);
     // CTAs per (query tile, head): as many as keep the launch within about two CTAs per SM (a wave),
     // so that short layers use every SM and long ones keep whole rows in one CTA; no more than
-    // a row has key tiles.  Clusters of four fill the wave with CTAs of up to a dozen tiles: there
-    // each CTA gets an SM to itself (by its shared-memory request), which takes the longest rows,
-    // started first, off the critical path (4 heads x 64, 1024 tokens: 53 -> 48 us for the layer;
-    // 4 x 128: 78 -> 66 us).
+    // a row has key tiles.
     int C = 1;
     while (C < 8 && 2 * C <= tiles && (long long)tiles * a.Hq * 2 * C <= 360) C *= 2;
-    const size_t smem = C == 4 ? (size_t)120 * 1024 : Shape<D>::kSmem;
+    // Clusters of two and four: each CTA gets an SM to itself (by its shared-memory request), which takes the longest rows,
+    // started first, off the critical path.  Attention with compaction, shared and alone, in us: two CTAs: 4 heads x 64, 1500
+    // tokens 60.8, 51.4, 2300 tokens 119, 79; 16 x 128, 400 tokens 50, 35; no shape of 13 slower.  Four: 4 x 64, 1024 tokens 35.2, 27.6;
+    // 4 x 128 61.0, 45.7; 2 x 64, 2300 64.5, 50.2; but where a CTA has one key tile or a third wave comes: 12 x 64, 200 tokens 12.3, 17.2;
+    // 8 x 64, 700 27.5, 35.6.  Eight (short chains): 4 x 64, 700 tokens 22.5, 32.5; 1 x 64, 2300 35.7, 41.7.
+    const long long ctas = (long long)tiles * a.Hq * C;
+    const bool alone = C == 2 || (C == 4 && (ctas <= 148 || (ctas <= 296 && tiles > C)));
+    const size_t smem = alone ? (size_t)120 * 1024 : Shape<D>::kSmem;
     cudaError_t e = cudaFuncSetAttribute(prefill_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          120 * 1024);
     if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "sparse_prefill: smem opt-in: %s", cudaGetErrorString(e));
