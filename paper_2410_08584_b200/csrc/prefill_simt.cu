@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(Shape<D>::kThreads)
 prefill_simt_kernel(LayerArgs a, const T *__restrict__ q, const T *__restrict__ k,
                     const T *__restrict__ v, const int32_t *__restrict__ idx,
                     const int32_t *__restrict__ k_dev, int k_max, T *__restrict__ out, int out_mode,
-                    T *__restrict__ kc, T *__restrict__ vc, int capacity, int32_t *__restrict__ len_out,
+                    T *__restrict__ kc, T *__restrict__ vc, int capacity, int32_t *__restrict__ len_out, int z0,
                     int32_t *status_word) {
     using S = Shape<D>;
     constexpr int TX = S::TX, kBN = S::kBN, NT = S::kThreads, KPT = S::KPT, CPT = S::CPT, QP = S::QP, PP = S::PP;
@@ -64,13 +64,13 @@ prefill_simt_kernel(LayerArgs a, const T *__restrict__ q, const T *__restrict__ 
     grid_launch_dependents();
     grid_dependency_wait(q, k, v, idx, k_dev);
     int n = *k_dev;
-    const int rank = blockIdx.x, C = gridDim.x, h = blockIdx.y, g = h / a.G;
+    const int rank = blockIdx.x, C = gridDim.x, h = blockIdx.y, z = z0 + (int)blockIdx.z, g = h / a.G;
     const int tid = threadIdx.x;
     if (n > k_max || n < 0) {
-        if (rank == 0 && h == 0 && blockIdx.z == 0 && tid == 0) report(status_word, ZIPVL_DEV_CAPACITY);
+        if (rank == 0 && h == 0 && z == 0 && tid == 0) report(status_word, ZIPVL_DEV_CAPACITY);
         n = n < 0 ? 0 : k_max;
     }
-    if (n == 0 && blockIdx.z == 0) {
+    if (n == 0 && z == 0) {
         // nothing kept: every row is a dropped token's row
         if (out_mode == ZIPVL_OUT_PADDED)
             for (long long e = rank * NT + tid; e < (long long)a.L * D; e += C * NT)
@@ -78,7 +78,7 @@ prefill_simt_kernel(LayerArgs a, const T *__restrict__ q, const T *__restrict__ 
         if (kc != nullptr && h == 0 && rank == 0 && tid == 0) *len_out = 0;
     }
     // the longest rows first; tiles past the kept set leave at once (the whole cluster together)
-    const int qt = (n + kBM - 1) / kBM - 1 - (int)blockIdx.z;
+    const int qt = (n + kBM - 1) / kBM - 1 - z;
     if (qt < 0) return;
     const int i0 = qt * kBM, i1 = min(n, i0 + kBM);
     const int n_kt = (i1 + kBN - 1) / kBN;              // key tiles up to the diagonal
@@ -349,7 +349,7 @@ prefill_simt_kernel(LayerArgs a, const T *__restrict__ q, const T *__restrict__ 
         }
         cl.sync();                                      // nobody leaves while its shared memory is read
     }
-    if (kF32 && kc != nullptr && h == 0 && blockIdx.z == 0 && rank == 0 && tid == 0) {
+    if (kF32 && kc != nullptr && h == 0 && z == 0 && rank == 0 && tid == 0) {
         *len_out = lim;
         if (n > capacity) report(status_word, ZIPVL_DEV_CAPACITY);
     }
@@ -361,7 +361,6 @@ zipvl_status run(const LayerArgs &a, const void *q, const void *k, const void *v
                  int capacity, int32_t *len_out, int32_t *status_word, cudaStream_t st) {
     static_assert(Shape<D>::kSmem <= 120 * 1024, "");
     const int tiles = (k_max + kBM - 1) / kBM;
-    if (tiles > 65535) return fail(ZIPVL_ERR_UNSUPPORTED, "sparse_prefill: k_max %d on the CUDA-core path", k_max);
     // CTAs per (query tile, head): as many as keep the launch within about two CTAs per SM (a wave),
     // so that short layers use every SM and long ones keep whole rows in one CTA; no more than
     // a row has key tiles.
@@ -378,11 +377,14 @@ zipvl_status run(const LayerArgs &a, const void *q, const void *k, const void *v
     cudaError_t e = cudaFuncSetAttribute(prefill_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          120 * 1024);
     if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "sparse_prefill: smem opt-in: %s", cudaGetErrorString(e));
-    e = launch_cluster(prefill_simt_kernel<T, D>, dim3(C, a.Hq, tiles), dim3(Shape<D>::kThreads), smem, st, C, a,
-                       (const T *)q, (const T *)k, (const T *)v, idx, k_dev, k_max, (T *)out, out_mode, (T *)kc,
-                       (T *)vc, capacity, len_out, status_word);
-    if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "sparse_prefill: launch: %s", cudaGetErrorString(e));
-    count_launches(1);
+    // (the grid's z ends at 65535, which a prompt of four million tokens has more tiles than)
+    for (int z0 = 0; z0 < tiles; z0 += 65535) {
+        e = launch_cluster(prefill_simt_kernel<T, D>, dim3(C, a.Hq, tiles - z0 < 65535 ? tiles - z0 : 65535),
+                           dim3(Shape<D>::kThreads), smem, st, C, a, (const T *)q, (const T *)k, (const T *)v, idx, k_dev, k_max,
+                           (T *)out, out_mode, (T *)kc, (T *)vc, capacity, len_out, z0, status_word);
+        if (e != cudaSuccess) return fail(ZIPVL_ERR_CUDA, "sparse_prefill: launch: %s", cudaGetErrorString(e));
+        count_launches(1);
+    }
     return check_launch("zipvl_sparse_prefill");
 }
 
