@@ -161,7 +161,7 @@ zipvl_status zipvl_score(const zipvl_layer *layer, const void *q, const void *k,
  *
  * acc, norm: device float[L], non-negative; a negative or NaN entry counts as zero in
  * the sums, ranks by its bit pattern and is reported as ZIPVL_DEV_BAD_VALUE.  Sums are
- * exact for scores below 2^18 (a column sum of attention is at most n_probe x n_q_heads).
+ * exact while a row's scores sum to less than 2^30 (columns of attention: n_probe x n_q_heads in all).
  * k_out: device int32[1].
  * idx: device int32[L].  kept_mass: device float[1] or NULL.
  * ws: zipvl_workspace_bytes(ZIPVL_OP_SELECT).  L <= 2^20.
@@ -407,8 +407,9 @@ zipvl_status zipvl_decode_quant_batch(const zipvl_decode_desc *desc, const void 
  * Same arguments and results as zipvl_decode, minus ws / ws_bytes.  Limit:
  * batch * n_q_heads * ceil(max_len / chunk) * (head_dim + 2) * 4 bytes must fit
  * in 8 MiB, where chunk is the number of cache rows the library gives one thread
- * block (from 32 to 512, growing with the problem; from 64 to 1536 for grouped query heads in 16-bit
- * storage) -- e.g. batch 16, 32 heads, head_dim 128 fits up to max_len 15872.  Larger problems are refused with
+ * block on the CUDA cores (32 to 512, growing with the problem; the tensor-core chunks of 16-bit storage,
+ * 64 to 1536 rows, need no more scratch than these wherever the limit is reached) -- e.g. batch 16,
+ * 32 heads, head_dim 128 fits up to max_len 15872.  Larger problems are refused with
  * ZIPVL_ERR_WORKSPACE and a message; use zipvl_decode with a workspace.
  *
  * The first call on each device looks up the array's device address (with that

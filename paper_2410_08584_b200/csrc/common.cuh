@@ -190,7 +190,7 @@ size_t decode_quant_ws_bytes(int B, int Hq, int Hkv, int D, int max_len);
 zipvl_status launch_decode_merge(int dtype, int D, int Hq, int B, int n_chunks, const float *ws,
                                  const int *lens, int32_t *seq_lens, void *out, cudaStream_t st,
                                  const zipvl_quant_cache *caches = nullptr);
-// Decode on the tensor cores (decode_mma.cu): 16-bit storage, head_dim 64 / 96 / 128, up to
+// Decode on the tensor cores (decode_mma.cu): 16-bit storage, head_dim 64 / 96 / 128, 1 to
 // 32 query heads per kv head.  partials, lens: pieces of the workspace (decode.cu).
 bool decode_mma_supported(const zipvl_decode_desc &d);
 int decode_mma_chunk(int B, int Hq, int Hkv, int D, int max_len);

@@ -8,8 +8,8 @@
 //   head (d elements) is read by d*sizeof/16 adjacent lanes with one 16-byte load
 //   each; the lanes of a row reduce the dot product by shuffles and keep an
 //   online softmax (base 2) for up to 8 query heads that share the kv head, so
-//   grouped-query attention still reads each cached byte once.  Four rows per
-//   lane group are in flight before any is consumed.
+//   grouped-query attention still reads each cached byte once.  Eight rows per
+//   lane group (four from three query heads on) are in flight before any is consumed.
 //   Append (Eq. 4): the CTA whose chunk holds row seq_lens[b] takes that row from
 //   k_new / v_new and stores it into the cache on the way.
 //   Each CTA leaves (m, l, o) for its chunk in the workspace.  The merge kernel

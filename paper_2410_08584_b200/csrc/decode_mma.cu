@@ -1,5 +1,5 @@
-// Grouped-query decode over the kept cache (Algorithm 2; Eq. 4 append, Eq. 5 attention of one query
-// token over the whole cache).  16-bit storage, head_dim 64, 96 or 128, 2 to 32 query heads per
+// Decode over the kept cache (Algorithm 2; Eq. 4 append, Eq. 5 attention of one query
+// token over the whole cache).  16-bit storage, head_dim 64, 96 or 128, 1 to 32 query heads per
 // key/value head, contiguous and paged caches.
 //
 // What bounds it: HBM, as long as a cached row costs few instructions.  With G query heads sharing a
@@ -8,7 +8,7 @@
 // rows go from memory to the registers that feed the MMA, no shared memory, no barrier, no role for
 // any warp but its own loop.  (A tcgen05 version with the G rows in a 128-row tile did 16 times
 // the arithmetic for G = 7 and needed a ring, producers and an issuer: 4.2 TB/s sustained on 16 requests of
-// 6K-30K rows, 28 heads on 4, against 5.9 here; one request of 732 rows: 8.6 -> 7.1 us.)
+// 6K-30K rows, 28 heads on 4, against 5.6 here; one request of 732 rows: 8.6 -> 7.1 us.)
 //   - S = K Q^T: A = 16 cached rows x 16 channels, B = 16 channels x 8 query heads.  The order
 //     of the 16 contraction indices is free as long as both operands share it, so a lane loads 16
 //     contiguous bytes of a row (four lanes 64) and they are the A registers of two MMAs;

@@ -609,12 +609,12 @@ select_kernel(int L, const float *__restrict__ acc, const float *__restrict__ no
 
 
 // ---------------------------------------------------------------------------------------
-// Rows of up to 4096 tokens: one CTA of 256 threads with the whole row in registers.
+// Rows of up to 4096 tokens: one CTA of 512 threads with the whole row in registers.
 //
-// Thread t owns positions 16t .. 16t+15 (four 16-byte loads per score vector), so the row is
+// Thread t owns positions 8t .. 8t+7 (two 16-byte loads per score vector), so the row is
 // read from memory once and the ascending emission is a walk over the thread's own registers.
 // A block-wide step costs a barrier plus its warp shuffles once per warp, so the CTA is kept
-// to eight warps and every phase to a few such steps; nothing loops over the row.
+// to sixteen warps and every phase to a few such steps; nothing loops over the row.
 //
 // The threshold searches are the ones described at the top of the file, with one change that
 // matters at this size: the histogram levels adapt to the data.  Level 1 spreads its 4096
@@ -628,13 +628,14 @@ select_kernel(int L, const float *__restrict__ acc, const float *__restrict__ no
 #define ZIPVL_SOLO_THREADS 512
 #endif
 constexpr int kSoloThreads = ZIPVL_SOLO_THREADS;
-constexpr int kSoloPer = kSoloMax / kSoloThreads;   // 16 positions per thread
+constexpr int kSoloPer = kSoloMax / kSoloThreads;   // 8 positions per thread
 constexpr int kSoloWarps = kSoloThreads / 32;
 
 struct SoloSmem {                      // dynamic shared memory
     // fixed-point sum of the budget score per bin as three words of 16-bit pieces (bits 0-15,
     // 16-31, 32 and up of each addend): three independent 32-bit adds without a carry to pass
-    // on; exact while a bin's pieces stay below 2^32, i.e. for scores below 2^18
+    // on; exact while the row's scores sum to less than 2^30 (the first two words hold 65536
+    // pieces of 16 bits)
     unsigned int sum16[3][kBins];
     unsigned int cnt[kBins];
     unsigned int cnt_r[kBins];         // level 1 of the ranking score (filled in the same walk)
@@ -689,7 +690,7 @@ __device__ __forceinline__ unsigned int solo_scan2(unsigned int v, SoloCtl &c, u
     return before + inc - v;
 }
 
-// block-wide (256 threads) exclusive prefix of a (count, sum) pair in thread order, and totals
+// block-wide exclusive prefix of a (count, sum) pair in thread order, and totals
 __device__ __forceinline__ void solo_scan(unsigned int vc, unsigned long long vs, SoloCtl &c,
                                           unsigned int *pc, unsigned long long *ps,
                                           unsigned int *tc = nullptr, unsigned long long *ts = nullptr) {
