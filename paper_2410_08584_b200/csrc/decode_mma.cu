@@ -32,9 +32,10 @@
 //     bytes per lane in flight.  The warps of a CTA take every fourth tile of its chunk and are merged
 //     through shared memory at the end; the chunks by decode_merge_kernel.
 //   - more than eight heads: two to four tiles of eight, whose chains, votes and merges run side by side.  Two
-//     CTAs fit an SM then, and from 25 heads of 128 channels on their eight warps no longer hide each other's
-//     latencies (issue slots 31% busy, tensor pipe 23%): 64 requests of 10K-20K rows on 2 kv heads, 24 heads 187 us
-//     (5.3 TB/s), 34 heads 212, 64 heads 273.
+//     CTAs fit an SM then, and their eight warps hold too few loads for HBM's latency: the rows of the step after
+//     the next are fetched into L2 (0.93 of the time over 68 shapes of more than a wave, 0.87 to 1.01; 0.99 over 112 in
+//     one wave).  From 25 heads of 128 channels on the warps no longer hide each other's latencies: 64 requests of
+//     10K-20K rows on 2 kv heads, 24 heads 167 us (5.9 TB/s), 34 heads 188, 64 heads 246.
 // Grid x is the kv head: the CTAs of one chunk run side by side and read whole rows of the cache together.
 // A tile is 16 rows, chunks start at multiples of 16 and pages are at least 16 rows, so a paged
 // cache costs one table look-up per tile.
@@ -103,6 +104,8 @@ __device__ __forceinline__ void store_row(void *p, const uint32_t (&w)[W]) {
     if constexpr (W == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
     else *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
 }
+
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 struct DmArgs {
     int Hq, Hkv, max_len, chunk, n_chunks;
@@ -248,6 +251,14 @@ decode_mma_kernel(DmArgs a) {
         const bool more = base + kWarps * 16 < c1;
         next_off = more ? tile_off(base + kWarps * 16) : -1;
         const int rows = c1 - base;
+        if (NT > 1 && rows > 2 * kWarps * 16) {      // the warp's tile after the next, into L2 (a lane: half a row of K and of V)
+            const int row = lane >> 1;
+            const long long far = kPaged ? tile_off(base + 2 * kWarps * 16) : off + 2 * kWarps * 16 * pitch;
+            if (far >= 0 && 2 * kWarps * 16 + row < rows) {
+                prefetch_l2(kb + far + row * pitch + (lane & 1) * (RB / 2));
+                prefetch_l2(vb + far + row * pitch + (lane & 1) * (RB / 2));
+            }
+        }
         // Eq. 4: the appended row, stored by the lanes that hold its pieces
         if (off >= 0 && new_row >= base && new_row < min(base + 16, c1)) {
             const int r = new_row - base;

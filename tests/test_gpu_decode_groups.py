@@ -70,3 +70,35 @@ def test_many_heads_on_more_than_a_wave(zipvl, G):
 def test_single_heads_of_64_channels(zipvl, n, L, H, dtype, page):
     """Either side of the lines between the two kernels: more than three requests, 100000 rows of heads, contiguous."""
     check_steps(zipvl, [L, 1, 17] + [max(0, L - 7 * i) for i in range(n - 3)], H, H, 64, dtype, page)
+
+
+@pytest.mark.parametrize("G", [9, 17, 32])
+@pytest.mark.parametrize("d,dtype", [(64, torch.float16), (96, torch.bfloat16), (128, torch.bfloat16)])
+@pytest.mark.parametrize("page", [0, 16])
+def test_rows_fetched_ahead(zipvl, G, d, dtype, page):
+    """Chunks of 512 rows whose ends lie around the tiles that a step fetches for the step after the next."""
+    check_steps(zipvl, [0, 127, 128, 129, 142, 143, 144, 145, 175, 192, 193, 511, 512, 513, 640, 641, 655] * 5, 2 * G, 2, d, dtype, page, steps=1)
+
+
+@pytest.mark.parametrize("G", [9, 17, 32])
+def test_page_outside_the_pool_ahead(zipvl, G):
+    """Its rows are left out and reported, as the tile of a step and as one that a step fetches ahead."""
+    z, B, L, d, page = zipvl, 80, 600, 64, 16
+    g = torch.Generator().manual_seed(G)
+    k, v = (torch.randn(L, 2, d, generator=g).to(torch.bfloat16) for _ in range(2))
+    q = torch.randn(B, 2 * G, d, generator=g).to(torch.bfloat16)
+    n = -(-L // page)
+    pools = [torch.cat([c, c.new_zeros(n * page - L, 2, d)]).view(n, page, 2, d).to(DEV) for c in (k, v)]
+    table = torch.arange(n, dtype=torch.int32).repeat(B, 1)
+    gone = [8, 9, 20]
+    table[:, gone] = torch.tensor([n, -1, n + 100000], dtype=torch.int32)
+    seq = torch.full((B,), L, dtype=torch.int32, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    desc = z.zipvl_decode_desc(B, 2 * G, 2, d, 0, 0.0)
+    out = z.zipvl_decode_paged(desc, q.to(DEV), None, None, *pools, table.to(DEV), torch.full_like(seq, n * page), seq, L, status=st)
+    rows = [r for r in range(L) if r // page not in gone]
+    kept = [to_np(c)[rows].reshape(-1).copy() for c in (k, v)]
+    want = oracle.decode_step(to_np(q), None, None, np.tile(kept[0], B), np.tile(kept[1], B),
+                              np.arange(B, dtype=np.int64) * kept[0].size, np.full(B, len(rows), np.int32), 2)
+    check_attention(to_np(out), want, torch.bfloat16)
+    assert st.item() & z.DEV_BAD_INDEX
